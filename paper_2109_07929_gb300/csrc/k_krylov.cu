@@ -29,7 +29,7 @@ constexpr int kThreads = 256;
 template <int KP>
 __device__ __forceinline__ void block_store_partials(double (&acc)[KP], int nk,
                                                      double* __restrict__ part, int b,
-                                                     int nblk) {
+                                                     int nblk, int vb) {
   __shared__ double red[kThreads / 32][KP];
   const int wv = threadIdx.x >> 5, l = threadIdx.x & 31;
   const double tot = warp_sum_scatter<KP>(acc);
@@ -39,34 +39,20 @@ __device__ __forceinline__ void block_store_partials(double (&acc)[KP], int nk,
     double s = 0.0;
 #pragma unroll
     for (int q = 0; q < kThreads / 32; ++q) s += red[q][threadIdx.x];
-    part[((size_t)b * 32 + threadIdx.x) * nblk + blockIdx.x] = s;
+    part[((size_t)b * 32 + threadIdx.x) * nblk + vb] = s;
     __threadfence();
   }
 }
 
-// True in every thread of the block that finished last among the nblk blocks of vector b
-// (its partial sums are then all visible); the counter is reset by the caller.
-__device__ __forceinline__ bool last_block(unsigned int* cnt, int b, int nblk) {
+// True in every thread of the block that finished last among the launch's blocks of vector
+// b (its partial sums are then all visible); the counter is reset by the caller.
+__device__ __forceinline__ bool last_block(unsigned int* cnt, int b) {
   __shared__ bool last;
   __syncthreads();
-  if (threadIdx.x == 0) last = (atomicAdd(&cnt[b], 1u) == (unsigned)nblk - 1);
+  if (threadIdx.x == 0) last = (atomicAdd(&cnt[b], 1u) == gridDim.x - 1);
   __syncthreads();
   if (last) __threadfence();
   return last;
-}
-
-// Fixed-order reduction of part[b][j][0..nblk) into h[b][j] = scale[j] * sum (j < nk),
-// warp w taking rows w, w + 8, ...
-__device__ __forceinline__ void block_reduce_rows(const double* __restrict__ part, int b,
-                                                  int nblk, int nk, double* __restrict__ h,
-                                                  const double* scale) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  for (int j = w; j < nk; j += kThreads / 32) {
-    double s = 0.0;
-    for (int t = l; t < nblk; t += 32) s += __ldcg(&part[((size_t)b * 32 + j) * nblk + t]);
-    s = warp_sum(s);
-    if (l == 0) h[(size_t)b * 32 + j] = scale ? s * scale[j] : s;
-  }
 }
 
 // h[b][j] = sum over blocks of part[b][j][:] for j < nk.
@@ -83,8 +69,17 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
   }
 }
 
+// The reductions below follow one summation order, whatever the launch shape: nblk blocks
+// of kThreads accumulators per vector (vec_nblk; the Jacobian
+// apply: residual_nblk), accumulator (v, t) adding the
+// entries v kThreads + t + k nblk kThreads in order; then a butterfly over each 32
+// accumulators, the warps of a block in order, and the blocks' partial sums by 32 lanes and
+// a butterfly.  Results (and with them the rounding of the BF16 preconditioner's inputs) do
+// not depend on how many accumulators a thread holds.
+
 // pass 3 (marked vectors only): partial dots <V_j, u> of the new vector u, reduced by the
-// last block into h2_j = s_j <V_j, u>.
+// last block into h2_j = s_j <V_j, u>.  Rarely does any work, so a launch has a quarter of
+// the summation's blocks, each taking them in turn.
 // ZS: the Newton step from V = 0, whose v_0 is stored in the first column of the top layer
 // only (the residual's sparse_f); its other entries are not read.
 template <int KP, bool ZS = false>
@@ -94,23 +89,26 @@ k_reorth_dots(const double* __restrict__ u, const double* __restrict__ V, size_t
               const VecCtl* __restrict__ ctl, unsigned int* cnt, double* h2, int ncols) {
   const int b = blockIdx.y;
   if (!ctl[b].gm_active || !ctl[b].reorth) return;
-  double acc[KP];
-#pragma unroll
-  for (int j = 0; j < KP; ++j) acc[j] = 0.0;
   const double* ub = u + (size_t)b * vstride;
   const double* Vb = V + (size_t)b * vstride;
   const int N2 = (int)n2;
   const int mn = N2 / 2, n = ncols;
-  for (int e = blockIdx.x * kThreads + threadIdx.x; e < N2; e += nblk * kThreads) {
-    const double x = ub[e];
-    const bool v0 = !ZS || (e < mn && e % n == 0);
+  for (int vb = blockIdx.x; vb < nblk; vb += gridDim.x) {
+    double acc[KP];
 #pragma unroll
-    for (int j = 0; j < KP; ++j)
-      if (j < nk && (!ZS || j > 0 || v0)) acc[j] = fma(Vb[(size_t)j * n2 + e], x, acc[j]);
+    for (int j = 0; j < KP; ++j) acc[j] = 0.0;
+    for (int e = vb * kThreads + threadIdx.x; e < N2; e += nblk * kThreads) {
+      const double x = ub[e];
+      const bool v0 = !ZS || (e < mn && e % n == 0);
+#pragma unroll
+      for (int j = 0; j < KP; ++j)
+        if (j < nk && (!ZS || j > 0 || v0)) acc[j] = fma(Vb[(size_t)j * n2 + e], x, acc[j]);
+    }
+    block_store_partials<KP>(acc, nk, part, b, nblk, vb);
+    __syncthreads();
   }
-  block_store_partials<KP>(acc, nk, part, b, nblk);
-  if (last_block(cnt, b, nblk)) {
-    block_reduce_rows(part, b, nblk, nk, h2, ctl[b].s);
+  if (last_block(cnt, b)) {
+    reduce_rows(part, b, nblk, nk, h2, ctl[b].s);
     if (threadIdx.x == 0) cnt[b] = 0;
   }
 }
@@ -118,97 +116,182 @@ k_reorth_dots(const double* __restrict__ u, const double* __restrict__ V, size_t
 // Passes 2 and 4: out <- w - sum_j hc_j v_j (the next, unnormalised basis vector, with
 // its BF16 copy for the tensor-core preconditioner), then the partial ||out||^2; the last
 // block of each vector runs the phase's control step (UpdPhase).
-template <int KP, bool ZS = false>
-__global__ void __launch_bounds__(kThreads)
+//
+// Bound: the FP64 pipe from nk = 3 on (nk + 1 FMAs per entry), HBM below.  Entries go in
+// pairs (16-byte loads; n2 is even, so every vector starts on a 16-byte boundary): half a
+// block takes one block of the summation, two accumulators per thread.  Two pairs are in
+// flight per thread, all their loads issued before the first store (out may alias w): G = 1
+// the next trip of the same accumulators, G = 2 (when the accumulators have one trip or
+// two) another block of the summation.  With one entry per thread and a butterfly per warp
+// the reduction and the coefficients took more FP64 instructions than the update itself
+// (256 x 256, 8 vectors, nk = 1 and 2: 34 and 38 us, now 16 and 20).
+// (layer, i, j) of a pair comes from one multiply-and-shift quotient.
+template <int KP, bool ZS, int G>
+__global__ void __launch_bounds__(kThreads, KP <= 4 ? 4 : (KP <= 8 ? 3 : 2))
 k_update_norm(int phase, const double* w, size_t wstride, const double* __restrict__ V,
               size_t vstride, size_t n2, int nk, const double* __restrict__ hc,
               double* __restrict__ part, int nblk, VecCtl* ctl, unsigned int* cnt,
               const double* __restrict__ h1, int restart, int32_t* host_flags, double* out,
-              size_t ostride, __nv_bfloat16* __restrict__ xbf, int mp, int np, int m, int n) {
+              size_t ostride, __nv_bfloat16* __restrict__ xbf, int mp, int np, int m, int n,
+              FastDiv by_n) {
   const int b = blockIdx.y;
   if (phase != UPD_PLAIN && (!ctl[b].gm_active || (phase == UPD_REORTH && !ctl[b].reorth)))
     return;
-  const double* sc = (phase != UPD_PLAIN) ? ctl[b].s : nullptr;
   double hj[KP];
 #pragma unroll
   for (int j = 0; j < KP; ++j)
-    hj[j] = (j < nk) ? hc[(size_t)b * 32 + j] * (sc ? sc[j] : 1.0) : 0.0;
-  const double* wb = w + (size_t)b * wstride;
-  double* ob = out + (size_t)b * ostride;
+    hj[j] = (j < nk) ? hc[(size_t)b * kHStride + 32 + j] : 0.0;
+  const double2* wb = reinterpret_cast<const double2*>(w + (size_t)b * wstride);
+  double2* ob = reinterpret_cast<double2*>(out + (size_t)b * ostride);
   const double* Vb = V + (size_t)b * vstride;
-  const size_t mn = n2 / 2;
-  double acc[1] = {0.0};
-  auto finish = [&](size_t e, double x) {
-    ob[e] = x;
-    if (xbf != nullptr) {
-      const int l = (e >= mn) ? 1 : 0;
-      const int cell = (int)(e - (size_t)l * mn);
-      const int i = cell / n, jj = cell - i * n;
-      xbf[(((size_t)b * 2 + l) * mp + i) * np + jj] = d2bf16_bits(x);
-    }
-    acc[0] = fma(x, x, acc[0]);
+  __nv_bfloat16* xb = xbf ? xbf + (size_t)b * 2 * mp * np : nullptr;
+  const uint32_t mn = (uint32_t)(n2 / 2), P = mn;      // P pairs = m n
+  const bool even = (n & 1) == 0;                      // no pair crosses a row
+  // position of entry e < 2 m n in the padded BF16 copy, and its column
+  auto pad = [&](uint32_t e, uint32_t& j) {
+    const uint32_t l = (e >= mn) ? 1u : 0u;
+    const uint32_t cell = e - l * mn;
+    const uint32_t i = by_n.quot(cell);
+    j = cell - i * (uint32_t)n;
+    return (l * (uint32_t)mp + i) * (uint32_t)np + j;
   };
-  // four elements per trip with all their loads issued before the first store (out may
-  // alias w, so the compiler cannot move loads of the next trip above the stores)
-  const size_t st = (size_t)nblk * kThreads;
-  size_t e = blockIdx.x * (size_t)kThreads + threadIdx.x;
-  // ZS: v_0 is stored (and nonzero) in the first column of the top layer only
-  auto v0 = [&](size_t e) { return !ZS || (e < mn && e % (size_t)n == 0); };
-  for (; e + 3 * st < n2; e += 4 * st) {
-    double x[4];
+  auto finish = [&](uint32_t p, double2 x, double (&acc)[2]) {
+    ob[p] = x;
+    if (xb != nullptr) {
+      uint32_t j;
+      const uint32_t o = pad(2 * p, j);
+      const __nv_bfloat16 b0 = d2bf16_bits(x.x), b1 = d2bf16_bits(x.y);
+      if (even) {
+        *reinterpret_cast<__nv_bfloat162*>(xb + o) = __nv_bfloat162(b0, b1);
+      } else {
+        xb[o] = b0;
+        xb[(j + 1 < (uint32_t)n) ? o + 1 : pad(2 * p + 1, j)] = b1;
+      }
+    }
+    acc[0] = fma(x.x, x.x, acc[0]);
+    acc[1] = fma(x.y, x.y, acc[1]);
+  };
+  // x -= hj_j V_j of pair p.  ZS: v_0 is stored (and nonzero) in the first column of the
+  // top layer only
+  auto sub = [&](int j, uint32_t p, double2& x) {
+    const double* vj = Vb + (size_t)j * n2;
+    if (ZS && j == 0) {
+      const uint32_t e = 2 * p;
+      if (e < mn && by_n.quot(e) * (uint32_t)n == e) x.x = fma(-hj[0], vj[e], x.x);
+      if (e + 1 < mn && by_n.quot(e + 1) * (uint32_t)n == e + 1)
+        x.y = fma(-hj[0], vj[e + 1], x.y);
+    } else {
+      const double2 v = reinterpret_cast<const double2*>(vj)[p];
+      x.x = fma(-hj[j], v.x, x.x);
+      x.y = fma(-hj[j], v.y, x.y);
+    }
+  };
+  auto one = [&](uint32_t p, double (&acc)[2]) {
+    double2 x = wb[p];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = wb[e + u * st];
+    for (int j = 0; j < KP; ++j)
+      if (j < nk) sub(j, p, x);
+    finish(p, x, acc);
+  };
+  auto two = [&](uint32_t p, uint32_t q, double (&accp)[2], double (&accq)[2]) {
+    double2 x = wb[p], y = wb[q];
 #pragma unroll
     for (int j = 0; j < KP; ++j)
       if (j < nk) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (!ZS || j > 0 || v0(e + u * st))
-            x[u] = fma(-hj[j], Vb[(size_t)j * n2 + e + u * st], x[u]);
+        sub(j, p, x);
+        sub(j, q, y);
       }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) finish(e + u * st, x[u]);
+    finish(p, x, accp);
+    finish(q, y, accq);
+  };
+  constexpr uint32_t kHalf = kThreads / 2;             // pairs of one block of the summation
+  const uint32_t half = threadIdx.x / kHalf;
+  const uint32_t vb0 = 2 * G * blockIdx.x + half;      // G = 2: also vb0 + 2
+  const uint32_t st = (uint32_t)nblk * kHalf;
+  double acc[G][2] = {};
+  uint32_t p = vb0 * kHalf + (threadIdx.x & (kHalf - 1));
+  if constexpr (G == 1) {
+    if (vb0 < (uint32_t)nblk) {
+      for (; p + st < P; p += 2 * st) two(p, p + st, acc[0], acc[0]);
+      if (p < P) one(p, acc[0]);
+    }
+  } else {
+    const bool second = vb0 + 2 < (uint32_t)nblk;
+    if (vb0 < (uint32_t)nblk) {
+      for (; p < P; p += st) {
+        const uint32_t q = p + 2 * kHalf;
+        if (second && q < P) two(p, q, acc[0], acc[1]);
+        else one(p, acc[0]);
+      }
+    }
   }
-  for (; e < n2; e += st) {
-    double x = wb[e];
-#pragma unroll
-    for (int j = 0; j < KP; ++j)
-      if (j < nk && (!ZS || j > 0 || v0(e))) x = fma(-hj[j], Vb[(size_t)j * n2 + e], x);
-    finish(e, x);
+  // the butterfly over 32 accumulators, which sit in 16 lanes (two each): its first levels
+  // halve what a lane holds, its last level joins the two
+  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
+  double t0 = acc[0][0], t1 = acc[0][1];
+  if constexpr (G == 2) {
+    const bool up = (lane & 8) != 0;
+    const double s0 = up ? acc[0][0] : acc[1][0], s1 = up ? acc[0][1] : acc[1][1];
+    t0 = (up ? acc[1][0] : acc[0][0]) + __shfl_xor_sync(0xffffffffu, s0, 8);
+    t1 = (up ? acc[1][1] : acc[0][1]) + __shfl_xor_sync(0xffffffffu, s1, 8);
   }
-  block_store_partials<1>(acc, 1, part, b, nblk);
+  constexpr int kFirst = (G == 2) ? 4 : 8;
+  {
+    const bool up = (lane & kFirst) != 0;
+    t0 = (up ? t1 : t0) + __shfl_xor_sync(0xffffffffu, up ? t0 : t1, kFirst);
+  }
+#pragma unroll
+  for (int o = kFirst / 2; o > 0; o >>= 1) t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+  t0 += __shfl_xor_sync(0xffffffffu, t0, kFirst);
+  __shared__ double red[G][2][kThreads / 32];
+  if ((lane & 7) == 0 && (G == 2 || (lane & 8) == 0))
+    red[G == 2 ? (lane >> 3) & 1 : 0][half][(wv & 3) * 2 + (lane >> 4)] = t0;
+  __syncthreads();
+  if (threadIdx.x < 2 * G) {
+    const int g = threadIdx.x >> 1, hf = threadIdx.x & 1;
+    const int vb = 2 * (G * (int)blockIdx.x + g) + hf;
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < kThreads / 32; ++q) s += red[g][hf][q];
+    if (vb < nblk) part[(size_t)b * 32 * nblk + vb] = s;
+    __threadfence();
+  }
   if (phase == UPD_PLAIN) return;
-  if (last_block(cnt, b, nblk)) {
-    __shared__ double hn2;
+  if (last_block(cnt, b)) {
+    __shared__ GsShared gs;
+    __shared__ double ps[kMaxVecBlocks];
+    for (int t = threadIdx.x; t < nblk; t += kThreads)
+      ps[t] = __ldcg(&part[(size_t)b * 32 * nblk + t]);
+    if (threadIdx.x == 0) cnt[b] = 0;
+    __syncthreads();
     if (threadIdx.x < 32) {
       double s = 0.0;
-      for (int t = threadIdx.x; t < nblk; t += 32) s += __ldcg(&part[((size_t)b * 32) * nblk + t]);
+      for (int t = threadIdx.x; t < nblk; t += 32) s += ps[t];
       s = warp_sum(s);
-      if (threadIdx.x == 0) hn2 = s;
+      if (threadIdx.x == 0) gs.hn2 = s;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      cnt[b] = 0;
-      gram_schmidt_control(ctl[b], b, phase, hn2, hc, h1, nk, restart, host_flags);
-    }
+    gram_schmidt_control(ctl[b], phase, hc + (size_t)b * kHStride, h1 + (size_t)b * kHStride, nk,
+                         restart, host_flags ? host_flags + b : nullptr, gs);
   }
-}
-
-// y = R^-1 g (upper triangular back substitution of the rotated Hessenberg matrix).
-__global__ void k_lsq(VecCtl* ctl) {
-  const int b = blockIdx.x;
-  VecCtl& c = ctl[b];
-  if (threadIdx.x != 0 || !c.newton_active) return;
-  lsq_solve(c);
 }
 
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f2d_bits(x); }
 
-// x <- x + sum_j y_j z_j over the finished cycle (Z in FP64 or FP32).
-template <typename ZT>
-__global__ void k_update_x(double* __restrict__ x, const ZT* __restrict__ Z,
-                           size_t zstride, size_t n2, const VecCtl* __restrict__ ctl) {
+__device__ __forceinline__ double2 widen2(const double* z, uint32_t p) {
+  return reinterpret_cast<const double2*>(z)[p];
+}
+__device__ __forceinline__ double2 widen2(const float* z, uint32_t p) {
+  const float2 v = reinterpret_cast<const float2*>(z)[p];
+  return make_double2(f2d_bits(v.x), f2d_bits(v.y));
+}
+
+// x <- x + sum_j y_j z_j over the finished cycle (Z in FP64 or FP32), entries in pairs
+// (W = 2, x on a 16-byte boundary) or one by one.  Bound: the FP64 pipe (k FMAs per entry).
+template <typename ZT, int W>
+__global__ void __launch_bounds__(kThreads)
+k_update_x(double* __restrict__ x, const ZT* __restrict__ Z, size_t zstride, size_t n2,
+           const VecCtl* __restrict__ ctl) {
   const int b = blockIdx.y;
   const VecCtl& c = ctl[b];
   if (!c.newton_active) return;
@@ -218,27 +301,40 @@ __global__ void k_update_x(double* __restrict__ x, const ZT* __restrict__ Z,
   __syncthreads();
   double* xb = x + (size_t)b * n2;
   const ZT* Zb = Z + (size_t)b * zstride;
-  // 32-bit element indices (n2 < 2^31), as in k_update_norm
-  const int N2 = (int)n2;
-  const int st = gridDim.x * blockDim.x;
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  for (; e + 3 * st < N2; e += 4 * st) {     // four independent elements per trip
-    double s[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) s[u] = xb[e + u * st];
-    const ZT* zj = Zb;
-    for (int j = 0; j < kd; ++j, zj += n2) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s[u] = fma(ys[j], widen(zj[e + u * st]), s[u]);
+  const uint32_t st = gridDim.x * kThreads, N = (uint32_t)(n2 / W);
+  uint32_t e = blockIdx.x * kThreads + threadIdx.x;
+  if constexpr (W == 2) {
+    double2* x2 = reinterpret_cast<double2*>(xb);
+    for (; e + st < N; e += 2 * st) {          // two independent pairs per trip
+      double2 s0 = x2[e], s1 = x2[e + st];
+      const ZT* zj = Zb;
+      for (int j = 0; j < kd; ++j, zj += n2) {
+        const double2 z0 = widen2(zj, e), z1 = widen2(zj, e + st);
+        s0.x = fma(ys[j], z0.x, s0.x);
+        s0.y = fma(ys[j], z0.y, s0.y);
+        s1.x = fma(ys[j], z1.x, s1.x);
+        s1.y = fma(ys[j], z1.y, s1.y);
+      }
+      x2[e] = s0;
+      x2[e + st] = s1;
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) xb[e + u * st] = s[u];
-  }
-  for (; e < N2; e += st) {
-    double s = xb[e];
-    const ZT* zj = Zb;
-    for (int j = 0; j < kd; ++j, zj += n2) s = fma(ys[j], widen(zj[e]), s);
-    xb[e] = s;
+    for (; e < N; e += st) {
+      double2 s0 = x2[e];
+      const ZT* zj = Zb;
+      for (int j = 0; j < kd; ++j, zj += n2) {
+        const double2 z0 = widen2(zj, e);
+        s0.x = fma(ys[j], z0.x, s0.x);
+        s0.y = fma(ys[j], z0.y, s0.y);
+      }
+      x2[e] = s0;
+    }
+  } else {
+    for (; e < N; e += st) {
+      double s = xb[e];
+      const ZT* zj = Zb;
+      for (int j = 0; j < kd; ++j, zj += n2) s = fma(ys[j], widen(zj[e]), s);
+      xb[e] = s;
+    }
   }
 }
 
@@ -322,7 +418,7 @@ int vec_nblk(size_t n2, int B) {
   size_t nb = (n2 + kThreads - 1) / kThreads;
   const size_t want = (kGridBlocks + B - 1) / (size_t)(B < 1 ? 1 : B);
   if (nb > want) nb = want;
-  if (nb > 608) nb = 608;
+  if (nb > kMaxVecBlocks) nb = kMaxVecBlocks;
   return nb < 1 ? 1 : (int)nb;
 }
 
@@ -331,27 +427,31 @@ void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
   k_reduce_dots<<<B, kThreads, 0, s>>>(part, nblk, nk, h, ctl);
 }
 
-#define MCA_KP_DISPATCH1(KERN, ZS_, nk, grid, ...)                             \
-  do {                                                                        \
-    if ((nk) <= 1) KERN<1, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__);       \
-    else if ((nk) <= 2) KERN<2, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__);  \
-    else if ((nk) <= 4) KERN<4, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__);  \
-    else if ((nk) <= 8) KERN<8, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__);  \
-    else if ((nk) <= 16) KERN<16, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__); \
-    else KERN<32, ZS_><<<grid, kThreads, 0, s>>>(__VA_ARGS__);                \
-  } while (0)
-#define MCA_KP_DISPATCH(KERN, zs, nk, grid, ...)                              \
-  do {                                                                        \
-    if (zs) MCA_KP_DISPATCH1(KERN, true, nk, grid, __VA_ARGS__);              \
-    else MCA_KP_DISPATCH1(KERN, false, nk, grid, __VA_ARGS__);                \
+#define MCA_KP_DISPATCH(nk, CALL)      \
+  do {                                 \
+    if ((nk) <= 1) CALL(1);            \
+    else if ((nk) <= 2) CALL(2);       \
+    else if ((nk) <= 4) CALL(4);       \
+    else if ((nk) <= 8) CALL(8);       \
+    else if ((nk) <= 16) CALL(16);     \
+    else CALL(32);                     \
   } while (0)
 
 void launch_reorth_dots(const double* u, const double* V, size_t vstride, size_t n2, int nk,
                         double* part, int nblk, int B, const VecCtl* ctl, unsigned int* cnt,
                         double* h2, cudaStream_t s, bool zs, int ncols) {
-  dim3 grid(nblk, B);
-  MCA_KP_DISPATCH(k_reorth_dots, zs, nk, grid, u, V, vstride, n2, nk, part, nblk, ctl, cnt, h2,
-                  ncols);
+  const dim3 grid((nblk + 3) / 4, B);
+#define MCA_CALL(KP_)                                                                        \
+  do {                                                                                       \
+    if (zs)                                                                                  \
+      k_reorth_dots<KP_, true><<<grid, kThreads, 0, s>>>(u, V, vstride, n2, nk, part, nblk,  \
+                                                         ctl, cnt, h2, ncols);               \
+    else                                                                                     \
+      k_reorth_dots<KP_, false><<<grid, kThreads, 0, s>>>(u, V, vstride, n2, nk, part, nblk, \
+                                                          ctl, cnt, h2, ncols);              \
+  } while (0)
+  MCA_KP_DISPATCH(nk, MCA_CALL);
+#undef MCA_CALL
 }
 
 void launch_update_norm(int phase, const double* w, size_t wstride, const double* V,
@@ -360,28 +460,48 @@ void launch_update_norm(int phase, const double* w, size_t wstride, const double
                         int restart, int32_t* host_flags, double* out, size_t ostride,
                         __nv_bfloat16* xbf, int mp, int np, int m, int n, cudaStream_t s,
                         bool zs) {
-  dim3 grid(nblk, B);
-  MCA_KP_DISPATCH(k_update_norm, zs, nk, grid, phase, w, wstride, V, vstride, n2, nk, hc, part,
-                  nblk, ctl, cnt, h1, restart, host_flags, out, ostride, xbf, mp, np, m, n);
+  // two blocks of the summation per block, or four when their accumulators see at most two
+  // entries each (then a thread would otherwise have one pair in flight)
+  const bool four = n2 <= 2 * (size_t)nblk * kThreads;
+  const dim3 grid(four ? (nblk + 3) / 4 : (nblk + 1) / 2, B);
+  const FastDiv by_n(n);
+#define MCA_CALL3(KP_, ZS_, G_)                                                             \
+  k_update_norm<KP_, ZS_, G_><<<grid, kThreads, 0, s>>>(                                    \
+      phase, w, wstride, V, vstride, n2, nk, hc, part, nblk, ctl, cnt, h1, restart,         \
+      host_flags, out, ostride, xbf, mp, np, m, n, by_n)
+#define MCA_CALL(KP_)                                                                       \
+  do {                                                                                      \
+    if (zs && four) MCA_CALL3(KP_, true, 2);                                                \
+    else if (zs) MCA_CALL3(KP_, true, 1);                                                   \
+    else if (four) MCA_CALL3(KP_, false, 2);                                                \
+    else MCA_CALL3(KP_, false, 1);                                                          \
+  } while (0)
+  MCA_KP_DISPATCH(nk, MCA_CALL);
+#undef MCA_CALL
+#undef MCA_CALL3
 }
 
 template <typename ZT>
-void lsq_update(double* x, const ZT* Z, size_t zstride, size_t n2, VecCtl* ctl, int B,
-                cudaStream_t s) {
-  k_lsq<<<B, 32, 0, s>>>(ctl);
-  int nb = (int)((n2 + kThreads - 1) / kThreads);
+void update_x(double* x, const ZT* Z, size_t zstride, size_t n2, VecCtl* ctl, int B,
+              cudaStream_t s) {
+  // one block per SM slot at most, four entries per thread at least
+  int nb = (int)((n2 + 4 * kThreads - 1) / (4 * kThreads));
   if (nb > 608) nb = 608;
-  k_update_x<ZT><<<dim3(nb, B), kThreads, 0, s>>>(x, Z, zstride, n2, ctl);
+  const dim3 grid(nb, B);
+  if ((reinterpret_cast<uintptr_t>(x) & 15) == 0)
+    k_update_x<ZT, 2><<<grid, kThreads, 0, s>>>(x, Z, zstride, n2, ctl);
+  else
+    k_update_x<ZT, 1><<<grid, kThreads, 0, s>>>(x, Z, zstride, n2, ctl);
 }
 
-void launch_lsq_update(double* x, const double* Z, size_t zstride, size_t n2, VecCtl* ctl,
+void launch_update_x(double* x, const double* Z, size_t zstride, size_t n2, VecCtl* ctl,
                        int B, cudaStream_t s) {
-  lsq_update(x, Z, zstride, n2, ctl, B, s);
+  update_x(x, Z, zstride, n2, ctl, B, s);
 }
 
-void launch_lsq_update(double* x, const float* Z, size_t zstride, size_t n2, VecCtl* ctl,
+void launch_update_x(double* x, const float* Z, size_t zstride, size_t n2, VecCtl* ctl,
                        int B, cudaStream_t s) {
-  lsq_update(x, Z, zstride, n2, ctl, B, s);
+  update_x(x, Z, zstride, n2, ctl, B, s);
 }
 
 }  // namespace mca

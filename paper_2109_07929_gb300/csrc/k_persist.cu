@@ -78,6 +78,7 @@ struct PSmem {
   int item;
   int err;
   uint32_t full_par, empty_par, pending;  // thread 0's pipeline state (bit s: stage s)
+  GsShared gs;
   double red[kWarps][32];
   double h1[32];
   double h2[32];
@@ -994,8 +995,8 @@ __device__ bool solve_item(const PersistShape& sh, const PersistItem& it, Work& 
       double hn2 = 0.0;
       MCA_PKP(update_phase, nk, sh, w, w.W, vnext, nk, S.h1, S, &hn2);
       if (!ok) return false;
-      if (threadIdx.x == 0)
-        gram_schmidt_control<false>(ctl, 0, UPD_FIRST, hn2, S.h1, S.h1, nk, restart, nullptr);
+      if (threadIdx.x == 0) S.gs.hn2 = hn2;
+      gram_schmidt_control(ctl, UPD_FIRST, S.h1, S.h1, nk, restart, nullptr, S.gs);
       proxy_fence_global();
       __syncthreads();
       clk.lap(PH_UPDATE);
@@ -1004,17 +1005,14 @@ __device__ bool solve_item(const PersistShape& sh, const PersistItem& it, Work& 
         if (!ok) return false;
         MCA_PKP(update_phase, nk, sh, w, vnext, vnext, nk, S.h2, S, &hn2);
         if (!ok) return false;
-        if (threadIdx.x == 0)
-          gram_schmidt_control<false>(ctl, 0, UPD_REORTH, hn2, S.h2, S.h1, nk, restart,
-                                      nullptr);
+        if (threadIdx.x == 0) S.gs.hn2 = hn2;
+        gram_schmidt_control(ctl, UPD_REORTH, S.h2, S.h1, nk, restart, nullptr, S.gs);
         proxy_fence_global();
         __syncthreads();
         clk.lap(PH_REORTH);
       }
       if (!ctl.gm_active) break;
     }
-    if (threadIdx.x == 0) lsq_solve(ctl);
-    __syncthreads();
     {
       const int kd = ctl.k_done;
       if (threadIdx.x < 32) S.h2[threadIdx.x] = (threadIdx.x < kd) ? ctl.y[threadIdx.x] : 0.0;

@@ -107,38 +107,33 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Block-wide sum of two values; result valid in thread 0.
-__device__ __forceinline__ void block_sum2(double& a, double& b) {
-  __shared__ double sa[kThreads / 32], sb[kThreads / 32];
-  a = warp_sum(a);
-  b = warp_sum(b);
+// Block-wide sums of N <= 4 values; results valid in thread 0.  The butterflies run as
+// warp_sum_scatter, in the same order (a butterfly per value took more FP64 instructions
+// than a cell's residual when a thread has one cell).
+template <int N>
+__device__ __forceinline__ void block_sums(double (&v)[N]) {
+  constexpr int KP = (N <= 1) ? 1 : ((N <= 2) ? 2 : 4);
+  __shared__ double red[kThreads / 32][KP];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) { sa[w] = a; sb[w] = b; }
+  double acc[KP];
+#pragma unroll
+  for (int q = 0; q < KP; ++q) acc[q] = (q < N) ? v[q] : 0.0;
+  const double tot = warp_sum_scatter<KP>(acc);
+  if (warp_scatter_writer<KP>(l)) red[w][warp_scatter_index<KP>(l)] = tot;
   __syncthreads();
   if (w == 0) {
-    a = (l < kThreads / 32) ? sa[l] : 0.0;
-    b = (l < kThreads / 32) ? sb[l] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
-  }
-}
-
-// Block-wide sum of three values; result valid in thread 0.
-__device__ __forceinline__ void block_sum3(double& a, double& b, double& c) {
-  __shared__ double sa[kThreads / 32], sb[kThreads / 32], sc[kThreads / 32];
-  a = warp_sum(a);
-  b = warp_sum(b);
-  c = warp_sum(c);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) { sa[w] = a; sb[w] = b; sc[w] = c; }
-  __syncthreads();
-  if (w == 0) {
-    a = (l < kThreads / 32) ? sa[l] : 0.0;
-    b = (l < kThreads / 32) ? sb[l] : 0.0;
-    c = (l < kThreads / 32) ? sc[l] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
+#pragma unroll
+    for (int q = 0; q < KP; ++q) acc[q] = (l < kThreads / 32) ? red[l][q] : 0.0;
+    const double all = warp_sum_scatter<KP>(acc);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      // the lane that holds value q
+      int src = 0;
+#pragma unroll
+      for (int c = 31; c >= 0; --c)
+        if (warp_scatter_index<KP>(c) == q) src = c;
+      v[q] = __shfl_sync(0xffffffffu, all, src);
+    }
   }
 }
 
@@ -363,10 +358,10 @@ __global__ void k_setup_vectors(Grid gr, const double* __restrict__ vin, VecCtl*
     const double v = vin[(size_t)b * gr.m + i];
     s += v * v;
   }
-  double dummy = 0.0;
-  block_sum2(s, dummy);
+  double v[1] = {s};
+  block_sums(v);
   if (threadIdx.x == 0) {
-    init_ctl(ctl[b], gr.g_src * sqrt(s), warm != 0);
+    init_ctl(ctl[b], gr.g_src * sqrt(v[0]), warm != 0);
   }
 }
 
@@ -434,12 +429,15 @@ k_residual(Grid gr, const double* __restrict__ gmap, const double* __restrict__ 
     }
   }
   sd += f2d_bits(sdf);
-  double sz = f2d_bits(ss);
-  block_sum3(sf, sd, sz);
+  constexpr int kRows = PAIR ? 3 : 2;
+  double v[kRows];
+  v[0] = sf;
+  v[1] = sd;
+  if constexpr (PAIR) v[2] = f2d_bits(ss);
+  block_sums(v);
   if (threadIdx.x == 0) {
-    part[((size_t)b * 32 + 0) * nblk + blockIdx.x] = sf;
-    part[((size_t)b * 32 + 1) * nblk + blockIdx.x] = sd;
-    if (PAIR) part[((size_t)b * 32 + 2) * nblk + blockIdx.x] = sz;
+#pragma unroll
+    for (int q = 0; q < kRows; ++q) part[((size_t)b * 32 + q) * nblk + blockIdx.x] = v[q];
   }
 }
 
@@ -578,17 +576,18 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
   }
   sd += f2d_bits(sdf);
   sf += f2d_bits(sfh) + f2d_bits(sfl);
-  double sz = f2d_bits(ss);
   if (__syncthreads_or(dnot32) && threadIdx.x == 0) atomicOr(&ctl[b].d64_next, 1);
-  if (PAIR)
-    block_sum3(sf, sd, sz);
-  else
-    block_sum2(sf, sd);
+  // sums (PAIR: also of the squared term sizes)
+  constexpr int kRows = PAIR ? 3 : 2;
+  double v[kRows];
+  v[0] = sf;
+  v[1] = sd;
+  if constexpr (PAIR) v[2] = f2d_bits(ss);
+  block_sums(v);
   __shared__ bool last;
   if (threadIdx.x == 0) {
-    part[((size_t)b * 32 + 0) * nblk + blockIdx.x] = sf;
-    part[((size_t)b * 32 + 1) * nblk + blockIdx.x] = sd;
-    if (PAIR) part[((size_t)b * 32 + 2) * nblk + blockIdx.x] = sz;
+#pragma unroll
+    for (int q = 0; q < kRows; ++q) part[((size_t)b * 32 + q) * nblk + blockIdx.x] = v[q];
     __threadfence();
     last = (atomicAdd(&cnt[b], 1u) == (unsigned)nblk - 1);
   }
@@ -597,7 +596,6 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
   __threadfence();
   // fixed-order sum over blocks: warp 0 -> ||F||^2, warp 1 -> sum(D), warp 2 -> the
   // squared term sizes (PAIR)
-  constexpr int kRows = PAIR ? 3 : 2;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __shared__ double tot[3];
   if (w < kRows) {
@@ -642,20 +640,6 @@ __global__ void k_init_basis(const double* __restrict__ F, double sign, double* 
   }
 }
 
-// Deterministic reduction of part[b][j][0..nblk) (j < nk) into h[b][j] by the whole
-// block (warp w sums rows w, w + 8, ...).
-__device__ __forceinline__ void block_reduce_rows(const double* __restrict__ part, int b,
-                                                  int nblk, int nk, double* __restrict__ h,
-                                                  const double* scale) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  for (int j = w; j < nk; j += kThreads / 32) {
-    double s = 0.0;
-    for (int t = l; t < nblk; t += 32) s += __ldcg(&part[((size_t)b * 32 + j) * nblk + t]);
-    s = warp_sum(s);
-    if (l == 0) h[(size_t)b * 32 + j] = scale ? s * scale[j] : s;
-  }
-}
-
 // K2 fused with the first classical Gram-Schmidt pass: w = J z for one cell (both
 // layers), then partial dots <V_j, w> for j < nk; the last block of each vector reduces
 // the partials into h.
@@ -663,12 +647,97 @@ __device__ __forceinline__ void block_reduce_rows(const double* __restrict__ par
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f2d_bits(x); }
 
-template <int KP, typename ZT, int AM, bool ZS = false>
+template <typename T>
+struct Vec2;
+template <>
+struct Vec2<double> { using type = double2; };
+template <>
+struct Vec2<float> { using type = float2; };
+
+// One cell of w = J z in the arithmetic AM from a = z_t, bb = z_b and their neighbours
+// (zero off the grid); jf, jl, iu, il: first / last column, first / last row.
+template <typename ZT, int AM>
+__device__ __forceinline__ void apply_cell(const Grid& gr, ZT a, ZT bb, ZT tl, ZT tr, ZT bu,
+                                           ZT bd, double Dd, bool jf, bool jl, bool iu, bool il,
+                                           bool dsplit, double& ot, double& ob) {
+  if constexpr (AM == kApplyPair) {
+    apply_pair(a, bb, tl, tr, bu, bd, Dd, jf ? gr.dt0f : (jl ? gr.dtlf : gr.dtmf),
+               jf ? gr.dt0l : (jl ? gr.dtll : gr.dtml), iu ? gr.db0f : (il ? gr.dblf : gr.dbmf),
+               iu ? gr.db0l : (il ? gr.dbll : gr.dbml), gr, ot, ob, dsplit);
+  } else if constexpr (AM == kApplyF32) {
+    // FP32 apply (z is FP32 here): the same formula, rounded to FP32, widened exactly
+    const float cpl = d2f_round(Dd) * (a - bb);
+    const float dt = jf ? gr.dt0f : (jl ? gr.dtlf : gr.dtmf);
+    const float db = iu ? gr.db0f : (il ? gr.dblf : gr.dbmf);
+    ot = f2d_bits(fmaf(dt, a, fmaf(-gr.gtf, tl + tr, cpl)));
+    ob = f2d_bits(fmaf(db, bb, fmaf(-gr.gbf, bu + bd, -cpl)));
+  } else {
+    const double av = widen(a), bv = widen(bb);
+    const double cpl = Dd * (av - bv);
+    const double dt = jf ? gr.dt0 : (jl ? gr.dtl : gr.dtm);
+    const double db = iu ? gr.db0 : (il ? gr.dbl : gr.dbm);
+    ot = fma(dt, av, fma(-gr.gt, widen(tl) + widen(tr), cpl));
+    ob = fma(db, bv, fma(-gr.gb, widen(bu) + widen(bd), -cpl));
+  }
+}
+
+// Sums of KP accumulators per parity over the 16 lanes of a half-warp, in the order of a
+// butterfly over 32 accumulators of which a lane holds two neighbours (acc[0], acc[1]):
+// the recursive halving of warp_sum_scatter for the first four levels, then the two
+// parities.  Returns the total of accumulator half_scatter_index<KP>(lane).
+template <int KP>
+__device__ __forceinline__ double half_sum_scatter(double (&acc)[2][KP]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int L = 0; L < 4; ++L) {
+    const int o = 8 >> L;
+    const int h = KP >> (L + 1);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (h >= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < KP / 2; ++i) {
+          if (i < h) {
+            const double send = up ? acc[q][i] : acc[q][i + h];
+            const double keep = up ? acc[q][i + h] : acc[q][i];
+            acc[q][i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        }
+      } else {
+        acc[q][0] += __shfl_xor_sync(0xffffffffu, acc[q][0], o);
+      }
+    }
+  }
+  return acc[0][0] + acc[1][0];
+}
+
+template <int KP>
+__device__ __forceinline__ int half_scatter_index(int lane) {
+  int j = 0;
+#pragma unroll
+  for (int L = 0; L < 4; ++L) {
+    const int h = KP >> (L + 1);
+    if (h >= 1 && (lane & (8 >> L))) j += h;
+  }
+  return j;
+}
+
+// The summation order is the one described in k_krylov.cu, with the cells for entries (a
+// cell adds its top layer's product, then its bottom layer's).
+// W = 2: two neighbouring cells of a row per thread and trip, with 16-byte (FP32 z: 8-byte)
+// loads and one quotient per pair (n even, every pointer on such a boundary: the launcher
+// checks); half a block takes one block of the summation.  W = 1: one cell per thread and
+// trip, any n and alignment, and long bases (nk > 8), whose accumulators fill the registers.
+// Bound: the FP64 pipe from nk = 2 on (2 nk FMAs per cell and the apply's own instructions),
+// HBM below.  1024 x 1024, 16 vectors, nk = 1: 170 us one cell per thread, 157 us in pairs;
+// 256 x 256, 8 vectors, first step: 13.0 and 8.7 us.
+template <int KP, typename ZT, int AM, bool ZS, int W>
 __global__ void __launch_bounds__(kThreads)
 k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
             size_t zstride, double* __restrict__ w, const double* __restrict__ V,
             size_t vstride, int nk, double* __restrict__ part, int nblk,
-            const VecCtl* __restrict__ ctl, unsigned int* cnt, double* h) {
+            const VecCtl* __restrict__ ctl, unsigned int* cnt, double* h, FastDiv by_n) {
   const int b = blockIdx.y;
   if (ctl != nullptr && !ctl[b].gm_active) return;
   // the pair apply skips the split of D when every entry is an FP32 number
@@ -681,83 +750,100 @@ k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
   double* wt = w + (size_t)b * n2;
   double* wb = wt + mn;
   const double* Vb_ = V + (size_t)b * vstride;
-  double acc[KP];
-#pragma unroll
-  for (int j = 0; j < KP; ++j) acc[j] = 0.0;
-  for (int c = blockIdx.x * kThreads + threadIdx.x; c < mn; c += nblk * kThreads) {
-    const int i = c / n;
+  double acc[W][KP] = {};
+  const int half = (W == 2) ? (int)threadIdx.x / (kThreads / 2) : 0;
+  const int vb = W * blockIdx.x + half;                 // block of the summation
+  const int lane_c = (W == 2) ? 2 * ((int)threadIdx.x & (kThreads / 2 - 1)) : (int)threadIdx.x;
+  const int c0 = (vb < nblk) ? vb * kThreads + lane_c : mn;
+  for (int c = c0; c < mn; c += nblk * kThreads) {
+    const int i = (int)by_n.quot((uint32_t)c);
     const int jj = c - i * n;
-    double ot, ob;
-    if constexpr (AM == kApplyPair) {
-      const bool f = (jj == 0), l = (jj == n - 1), u = (i == 0), dn = (i == m - 1);
-      apply_pair(zt[c], zb[c], f ? 0.f : (float)zt[c - 1], l ? 0.f : (float)zt[c + 1],
-                 u ? 0.f : (float)zb[c - n], dn ? 0.f : (float)zb[c + n], Db[c],
-                 f ? gr.dt0f : (l ? gr.dtlf : gr.dtmf), f ? gr.dt0l : (l ? gr.dtll : gr.dtml),
-                 u ? gr.db0f : (dn ? gr.dblf : gr.dbmf), u ? gr.db0l : (dn ? gr.dbll : gr.dbml),
-                 gr, ot, ob, dsplit);
-    } else if constexpr (AM == kApplyF32) {
-      // FP32 apply (z is FP32 here): the same formula, rounded to FP32, widened exactly
-      const float a = zt[c], bb = zb[c];
-      const float cpl = d2f_round(Db[c]) * (a - bb);
-      const float dt = (jj == 0) ? gr.dt0f : ((jj == n - 1) ? gr.dtlf : gr.dtmf);
-      const float db = (i == 0) ? gr.db0f : ((i == m - 1) ? gr.dblf : gr.dbmf);
-      const float tl = (jj > 0) ? (float)zt[c - 1] : 0.f;
-      const float tr = (jj < n - 1) ? (float)zt[c + 1] : 0.f;
-      const float bu = (i > 0) ? (float)zb[c - n] : 0.f;
-      const float bd = (i < m - 1) ? (float)zb[c + n] : 0.f;
-      ot = f2d_bits(fmaf(dt, a, fmaf(-gr.gtf, tl + tr, cpl)));
-      ob = f2d_bits(fmaf(db, bb, fmaf(-gr.gbf, bu + bd, -cpl)));
-    } else {
-      const double a = widen(zt[c]), bb = widen(zb[c]);
-      const double cpl = Db[c] * (a - bb);
-      const double dt = (jj == 0) ? gr.dt0 : ((jj == n - 1) ? gr.dtl : gr.dtm);
-      const double db = (i == 0) ? gr.db0 : ((i == m - 1) ? gr.dbl : gr.dbm);
-      const double tl = (jj > 0) ? widen(zt[c - 1]) : 0.0;
-      const double tr = (jj < n - 1) ? widen(zt[c + 1]) : 0.0;
-      const double bu = (i > 0) ? widen(zb[c - n]) : 0.0;
-      const double bd = (i < m - 1) ? widen(zb[c + n]) : 0.0;
-      ot = fma(dt, a, fma(-gr.gt, tl + tr, cpl));
-      ob = fma(db, bb, fma(-gr.gb, bu + bd, -cpl));
-    }
-    wt[c] = ot;
-    wb[c] = ob;
-    if (V != nullptr) {
+    const bool iu = (i == 0), il = (i == m - 1);
+    if constexpr (W == 2) {
+      using Z2 = typename Vec2<ZT>::type;
+      const Z2 none{ZT(0), ZT(0)};
+      const Z2 a = *reinterpret_cast<const Z2*>(zt + c), q = *reinterpret_cast<const Z2*>(zb + c);
+      const Z2 u = iu ? none : *reinterpret_cast<const Z2*>(zb + c - n);
+      const Z2 d = il ? none : *reinterpret_cast<const Z2*>(zb + c + n);
+      const ZT tl = (jj == 0) ? ZT(0) : zt[c - 1];
+      const ZT tr = (jj + 2 == n) ? ZT(0) : zt[c + 2];
+      const double2 Dd = *reinterpret_cast<const double2*>(Db + c);
+      double2 ot, ob;
+      apply_cell<ZT, AM>(gr, a.x, q.x, tl, a.y, u.x, d.x, Dd.x, jj == 0, false, iu, il, dsplit,
+                         ot.x, ob.x);
+      apply_cell<ZT, AM>(gr, a.y, q.y, a.x, tr, u.y, d.y, Dd.y, false, jj + 2 == n, iu, il,
+                         dsplit, ot.y, ob.y);
+      *reinterpret_cast<double2*>(wt + c) = ot;
+      *reinterpret_cast<double2*>(wb + c) = ob;
+      if (V != nullptr) {
 #pragma unroll
-      for (int j = 0; j < KP; ++j) {
-        if (j < nk) {
-          const double* vj = Vb_ + (size_t)j * n2;
-          if (ZS && j == 0) {            // v_0 of the zero state: first top column only
-            if (jj == 0) acc[0] = fma(vj[c], ot, acc[0]);
-          } else {
-            acc[j] = fma(vj[c], ot, acc[j]);
-            acc[j] = fma(vj[mn + c], ob, acc[j]);
+        for (int j = 0; j < KP; ++j) {
+          if (j < nk) {
+            const double* vj = Vb_ + (size_t)j * n2 + c;
+            if (ZS && j == 0) {          // v_0 of the zero state: first top column only
+              if (jj == 0) acc[0][0] = fma(vj[0], ot.x, acc[0][0]);
+            } else {
+              const double2 vt = *reinterpret_cast<const double2*>(vj);
+              const double2 vb2 = *reinterpret_cast<const double2*>(vj + mn);
+              acc[0][j] = fma(vb2.x, ob.x, fma(vt.x, ot.x, acc[0][j]));
+              acc[1][j] = fma(vb2.y, ob.y, fma(vt.y, ot.y, acc[1][j]));
+            }
+          }
+        }
+      }
+    } else {
+      const bool jf = (jj == 0), jl = (jj == n - 1);
+      double ot, ob;
+      apply_cell<ZT, AM>(gr, zt[c], zb[c], jf ? ZT(0) : zt[c - 1], jl ? ZT(0) : zt[c + 1],
+                         iu ? ZT(0) : zb[c - n], il ? ZT(0) : zb[c + n], Db[c], jf, jl, iu, il,
+                         dsplit, ot, ob);
+      wt[c] = ot;
+      wb[c] = ob;
+      if (V != nullptr) {
+#pragma unroll
+        for (int j = 0; j < KP; ++j) {
+          if (j < nk) {
+            const double* vj = Vb_ + (size_t)j * n2 + c;
+            if (ZS && j == 0) {
+              if (jf) acc[0][0] = fma(vj[0], ot, acc[0][0]);
+            } else {
+              acc[0][j] = fma(vj[mn], ob, fma(vj[0], ot, acc[0][j]));
+            }
           }
         }
       }
     }
   }
   if (V == nullptr) return;
-  __shared__ double red[kThreads / 32][KP];
+  __shared__ double red[W][kThreads / 32][KP];
   const int wv = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const double tot = warp_sum_scatter<KP>(acc);
-  if (warp_scatter_writer<KP>(l)) red[wv][warp_scatter_index<KP>(l)] = tot;
+  if constexpr (W == 2) {
+    const double tot = half_sum_scatter<KP>(acc);
+    if ((l & (16 / KP - 1)) == 0)
+      red[half][(wv & 3) * 2 + (l >> 4)][half_scatter_index<KP>(l)] = tot;
+  } else {
+    const double tot = warp_sum_scatter<KP>(acc[0]);
+    if (warp_scatter_writer<KP>(l)) red[0][wv][warp_scatter_index<KP>(l)] = tot;
+  }
   __syncthreads();
-  if (threadIdx.x < nk && threadIdx.x < KP) {
+  if (threadIdx.x < W * KP) {
+    const int hf = threadIdx.x / KP, j = threadIdx.x - hf * KP;
+    const int v = W * blockIdx.x + hf;
     double s = 0.0;
 #pragma unroll
-    for (int q = 0; q < kThreads / 32; ++q) s += red[q][threadIdx.x];
-    part[((size_t)b * 32 + threadIdx.x) * nblk + blockIdx.x] = s;
+    for (int q = 0; q < kThreads / 32; ++q) s += red[hf][q][j];
+    if (j < nk && v < nblk) part[((size_t)b * 32 + j) * nblk + v] = s;
     __threadfence();
   }
   if (cnt == nullptr) return;
   __shared__ bool last;
   __syncthreads();
-  if (threadIdx.x == 0) last = (atomicAdd(&cnt[b], 1u) == (unsigned)nblk - 1);
+  if (threadIdx.x == 0) last = (atomicAdd(&cnt[b], 1u) == gridDim.x - 1);
   __syncthreads();
   if (!last) return;
   __threadfence();
   // the stored basis is unnormalised: <v_j, w> = s_j <V_j, w>
-  block_reduce_rows(part, b, nblk, nk, h, ctl ? ctl[b].s : nullptr);
+  reduce_rows(part, b, nblk, nk, h, ctl[b].s);
   if (threadIdx.x == 0) cnt[b] = 0;
 }
 
@@ -781,12 +867,11 @@ __global__ void k_outputs(Grid gr, const double* __restrict__ vin, const double*
     s_out += io;
     s_leak += gr.g_bt * Vb[j];
   }
-  block_sum2(s_in, s_abs);
-  __syncthreads();
-  block_sum2(s_out, s_leak);
+  double v[4] = {s_in, s_abs, s_out, s_leak};
+  block_sums(v);
   if (threadIdx.x == 0) {
-    const double bal = s_in - s_out - s_leak;
-    kcl[b] = (s_abs > 0.0) ? fabs(bal) / s_abs : 0.0;
+    const double bal = v[0] - v[2] - v[3];
+    kcl[b] = (v[1] > 0.0) ? fabs(bal) / v[1] : 0.0;
   }
 }
 
@@ -860,17 +945,23 @@ void spmv_dots(const Grid& gr, const double* D, const ZT* z, size_t zstride, dou
                const VecCtl* ctl, unsigned int* cnt, double* h, cudaStream_t s) {
   // z: the vector of batch entry 0, later entries zstride doubles apart; V: basis vector
   // 0 of batch entry 0 (nk vectors N2 apart, entries vstride apart), or NULL.
-  dim3 grid(nblk, B);
-#define MCA_SPMV(KP_)                                                                      \
-  k_spmv_dots<KP_, ZT, AM, ZS><<<grid, kThreads, 0, s>>>(gr, D, z, zstride, w, V, vstride, nk, \
-                                                      part, nblk, ctl, cnt, h)
+  // pairs of cells: every row starts on a pair, and every array on a 16-byte boundary
+  auto on = [](const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
+  const bool two = (gr.n & 1) == 0 && on(D, 16) && on(w, 16) && on(V, 16) &&
+                   on(z, 2 * sizeof(ZT)) && (zstride & 1) == 0 && (vstride & 1) == 0;
+  const FastDiv by_n(gr.n);
+#define MCA_SPMV1(KP_, W_)                                                                   \
+  k_spmv_dots<KP_, ZT, AM, ZS, W_><<<dim3((nblk + W_ - 1) / W_, B), kThreads, 0, s>>>(       \
+      gr, D, z, zstride, w, V, vstride, nk, part, nblk, ctl, cnt, h, by_n)
+#define MCA_SPMV(KP_) do { if (two) MCA_SPMV1(KP_, 2); else MCA_SPMV1(KP_, 1); } while (0)
   if (nk <= 1) MCA_SPMV(1);
   else if (nk <= 2) MCA_SPMV(2);
   else if (nk <= 4) MCA_SPMV(4);
   else if (nk <= 8) MCA_SPMV(8);
-  else if (nk <= 16) MCA_SPMV(16);
-  else MCA_SPMV(32);
+  else if (nk <= 16) MCA_SPMV1(16, 1);
+  else MCA_SPMV1(32, 1);
 #undef MCA_SPMV
+#undef MCA_SPMV1
 }
 
 void launch_spmv_dots(const Grid& gr, const double* D, const double* z, size_t zstride,

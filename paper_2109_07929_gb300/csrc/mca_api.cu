@@ -326,8 +326,8 @@ int alloc_workspace(mca_handle* h) {
     MCA_TRY(dalloc(h, &h->Z, B * h->restart * n2));
   MCA_TRY(dalloc(h, &h->W, B * n2));
   MCA_TRY(dalloc(h, &h->part, B * 32 * MCA_NPART));
-  MCA_TRY(dalloc(h, &h->h1, B * 32));
-  MCA_TRY(dalloc(h, &h->h2, B * 32));
+  MCA_TRY(dalloc(h, &h->h1, B * kHStride));
+  MCA_TRY(dalloc(h, &h->h2, B * kHStride));
   MCA_TRY(dalloc(h, &h->vinbuf[0], B * h->m));
   MCA_TRY(dalloc(h, &h->vinbuf[1], B * h->m));
   h->vin = h->vinbuf[0];
@@ -867,10 +867,10 @@ int solve_pass(mca_handle* h, int B, cudaStream_t s, bool from_guess = false) {
     MCA_TRY(gmres_cycle(h, h->D, B, s, f32));
     t0 = prof_begin(h, s);
     if (tc)
-      launch_lsq_update(h->x, h->Z32, zstride, h->n2, h->ctl, B, s);
+      launch_update_x(h->x, h->Z32, zstride, h->n2, h->ctl, B, s);
     else
-      launch_lsq_update(h->x, h->Z, zstride, h->n2, h->ctl, B, s);
-    count_launches(2);
+      launch_update_x(h->x, h->Z, zstride, h->n2, h->ctl, B, s);
+    count_launches(1);
     double kbar = 0.0;
     if (h->prof_on) {
       int c = 0;
@@ -1794,10 +1794,10 @@ int mca_gmres_solve(mca_handle* h, const double* D, const double* a, const doubl
     count_launches(3);
     MCA_TRY(gmres_cycle(h, D, nvec, s));
     if (tc)
-      launch_lsq_update(dx, h->Z32, zstride, n2, h->ctl, nvec, s);
+      launch_update_x(dx, h->Z32, zstride, n2, h->ctl, nvec, s);
     else
-      launch_lsq_update(dx, h->Z, zstride, n2, h->ctl, nvec, s);
-    count_launches(2);
+      launch_update_x(dx, h->Z, zstride, n2, h->ctl, nvec, s);
+    count_launches(1);
     MCA_CUDA_TRY(cudaGetLastError());
     MCA_CUDA_TRY(cudaMemcpyAsync(h->ctl_host.data(), h->ctl, (size_t)nvec * sizeof(VecCtl),
                                  cudaMemcpyDeviceToHost, s));

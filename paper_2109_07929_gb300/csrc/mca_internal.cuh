@@ -166,6 +166,24 @@ __device__ __forceinline__ bool warp_scatter_writer(int lane) {
   return (lane & (32 / KP - 1)) == 0;
 }
 
+// Quotient x / d for x < 2^31 by one wide multiplication and a shift (d >= 1), with
+// mul = floor(2^(31 + l) / d) + 1, 2^(l-1) < d <= 2^l: mul d exceeds 2^(31 + l) by at most
+// d <= 2^l, an error of less than 1 / d in x mul / 2^(31 + l).  (A 32-bit division takes
+// about twenty instructions; the vector kernels divide once per pair of entries.)
+struct FastDiv {
+  uint32_t mul;
+  int shift;
+  explicit FastDiv(int d) {
+    int l = 0;
+    while ((1 << l) < d) ++l;
+    shift = 31 + l;
+    mul = (uint32_t)((1ull << shift) / (unsigned long long)d + 1ull);
+  }
+  __host__ __device__ __forceinline__ uint32_t quot(uint32_t x) const {
+    return (uint32_t)(((unsigned long long)x * mul) >> shift);
+  }
+};
+
 // ---------------------------------------------------------------- kernels (launchers)
 // stencil / residual / Jacobian (k_stencil.cu)
 // warm: the states are a caller's guess (the first forcing term then follows
@@ -242,6 +260,10 @@ int residual_nblk(int mn, int B = 1);
 constexpr int kResidualMaxBlocks = 608;
 // Krylov (k_krylov.cu)
 int vec_nblk(size_t n2, int B = 1);
+constexpr int kMaxVecBlocks = 608;   // vec_nblk() never exceeds this
+// Gram-Schmidt coefficients of a vector: h_j at j < 32, s_j h_j (the factors of the stored,
+// unnormalised basis vectors in the update pass) at 32 + j.
+constexpr int kHStride = 64;
 void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
                         const VecCtl* ctl, cudaStream_t s);
 // pass 2: w -= V h1, partial dots <V_j, w>; the last block reduces them into h2.
@@ -267,10 +289,10 @@ void launch_update_norm(int phase, const double* w, size_t wstride, const double
                         int restart, int32_t* host_flags, double* out, size_t ostride,
                         __nv_bfloat16* xbf, int mp, int np, int m, int n, cudaStream_t s,
                         bool zs = false);
-void launch_lsq_update(double* x, const double* Z, size_t zstride, size_t n2, VecCtl* ctl,
-                       int B, cudaStream_t s);
-void launch_lsq_update(double* x, const float* Z, size_t zstride, size_t n2, VecCtl* ctl,
-                       int B, cudaStream_t s);
+void launch_update_x(double* x, const double* Z, size_t zstride, size_t n2, VecCtl* ctl, int B,
+                     cudaStream_t s);
+void launch_update_x(double* x, const float* Z, size_t zstride, size_t n2, VecCtl* ctl, int B,
+                     cudaStream_t s);
 // first = 1: remember beta = ||rhs|| and stop at rtol * beta; first = 0 (a restart): keep
 // the tolerance of the first cycle.
 void launch_gmres_init(const double* part_norm, int nblk, VecCtl* ctl, int B, double rtol,

@@ -274,52 +274,6 @@ __device__ void newton_control(VecCtl& c, double sf, double sd, int mn, const So
   __threadfence_system();
 }
 
-// Givens rotation of Hessenberg column k (h = h1 + h2, h2 may be NULL; h_{k+1,k} =
-// sqrt(hn2)), residual
-// estimate |g_{k+1}| and the stop test of the GMRES cycle.  One thread.
-// kL2: the h arrays were written by other blocks (read through L2); otherwise plain loads
-// (the persistent kernel keeps them in its own CTA's shared memory).
-template <bool kL2 = true>
-__device__ void givens_column(VecCtl& c, int b, double hn2, const double* __restrict__ h1,
-                              const double* __restrict__ h2, int k, int restart,
-                              int32_t* host_flags) {
-  auto ldh = [](const double* p) { return kL2 ? __ldcg(p) : *p; };
-  const int ld = MCA_KMAX + 1;
-  double* col = c.H + (size_t)k * ld;
-  for (int j = 0; j <= k; ++j)
-    col[j] = ldh(&h1[(size_t)b * 32 + j]) + (h2 ? ldh(&h2[(size_t)b * 32 + j]) : 0.0);
-  const double hk1 = sqrt(hn2);
-  col[k + 1] = hk1;
-  for (int j = 0; j < k; ++j) {
-    const double t = c.cs[j] * col[j] + c.sn[j] * col[j + 1];
-    col[j + 1] = -c.sn[j] * col[j] + c.cs[j] * col[j + 1];
-    col[j] = t;
-  }
-  const double rho = hypot(col[k], col[k + 1]);
-  double cs = 1.0, sn = 0.0;
-  if (rho > 0.0) {
-    cs = col[k] / rho;
-    sn = col[k + 1] / rho;
-  }
-  c.cs[k] = cs;
-  c.sn[k] = sn;
-  col[k] = rho;
-  col[k + 1] = 0.0;
-  c.g[k + 1] = -sn * c.g[k];
-  c.g[k] = cs * c.g[k];
-  const double res = fabs(c.g[k + 1]);
-  c.res_est = res;
-  c.k_done = k + 1;
-  c.gmres_iters += 1;
-  c.inv_h = (hk1 > 0.0) ? 1.0 / hk1 : 0.0;
-  c.s[k + 1] = c.inv_h;
-  const bool stop = !(res > c.tol_abs) || (k + 1 >= restart) || !(hk1 > 0.0) ||
-                    !(rho > 0.0) || !isfinite(res);
-  if (stop) c.gm_active = 0;
-  if (host_flags) host_flags[b] = c.gm_active;
-  __threadfence_system();
-}
-
 // Control block of one vector at the start of a solve: ||Y|| = yn and the counters; a
 // zero or non-finite input ends the solve at once.
 __device__ __forceinline__ void init_ctl(VecCtl& c, double yn, bool warm) {
@@ -351,57 +305,159 @@ __device__ __forceinline__ void init_ctl(VecCtl& c, double yn, bool warm) {
   }
 }
 
+// Shared-memory scratch of gram_schmidt_control.
+struct GsShared {
+  double hn2;                  // squared norm of the new vector (in)
+  double est, rho2;            // warp 2's orthogonality estimate
+};
+
 // Gram-Schmidt step control of one vector after an update pass (phase UPD_FIRST or
-// UPD_REORTH, see k_krylov.cu) for the new vector of squared norm hn2.  hc: the pass's
-// coefficients (h1 after the first pass, h2 after the second), h1: the first pass's.
+// UPD_REORTH, see k_krylov.cu), by the whole block (at least three warps; every thread
+// calls it; the block synchronises here before S.hn2, written by any of its threads, is
+// read).  hc: the pass's coefficients (h1 after the first pass, h2 after the second), h1:
+// the first pass's; both of nk = k + 1 entries, readable by the block.
 // UPD_FIRST estimates the loss of orthogonality of the new vector and either marks the
-// vector for the second pass or finishes Hessenberg column nk-1; UPD_REORTH finishes it with
-// h1 + h2.  One thread.  kL2: the coefficients were written by other blocks.
-template <bool kL2 = true>
-__device__ void gram_schmidt_control(VecCtl& c, int b, int phase, double hn2,
-                                     const double* __restrict__ hc,
-                                     const double* __restrict__ h1, int nk, int restart,
-                                     int32_t* host_flags) {
-  const int k = nk - 1;
-  const double grow = sqrt((double)nk) * c.orth;
-  if (phase == UPD_FIRST) {
-    double proj = 0.0;                      // |h1|^2 = |w|^2 - |u|^2
-    for (int j = 0; j < nk; ++j) {
-      const double t = kL2 ? __ldcg(&hc[(size_t)b * 32 + j]) : hc[(size_t)b * 32 + j];
-      proj = fma(t, t, proj);
+// vector for the second pass or finishes Hessenberg column k; UPD_REORTH finishes it with
+// h1 + h2.  Finishing a column: Givens rotations, residual estimate |g_{k+1}|, the stop
+// test of the GMRES cycle, and on a stop the least-squares solution y.
+//
+// An FP64 instruction has the latency of a warp's whole turn on the FP64 pipe here, and a
+// square root or a quotient is a chain of about ten, so one thread doing all this in order
+// took 6 us (32 x 32 crossbar: 10.1 us for an update pass whose data takes 4).  Warp 1
+// rotates the column (which needs only h) while warp 0 sums the norm, lanes take the three
+// quotients of the rotation side by side, and warp 2 makes the estimate.
+__device__ __noinline__ void gram_schmidt_control(VecCtl& c, int phase, const double* hc,
+                                                  const double* h1, int nk, int restart,
+                                                  int32_t* host_flag, GsShared& S) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  const int k = nk - 1, ld = MCA_KMAX + 1;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  double colk = 0.0, gk = 0.0, proj = 0.0, orth = 0.0, wn2 = 0.0, orth1 = 0.0;
+  if (w == 1) {
+    double col = 0.0, cs = 1.0, sn = 0.0, mine = 0.0;
+    if (l < nk) col = hc[l];
+    if (phase == UPD_REORTH && l < nk) col = h1[l] + col;
+    if (l < k) {
+      cs = c.cs[l];
+      sn = c.sn[l];
     }
-    const double rho = (hn2 > 0.0) ? sqrt(hn2 / (hn2 + proj)) : 0.0;
-    const double est = (grow + 4.0 * nk * kEps) / rho;
-    if (hn2 > 0.0 && !(est <= kOrthTol)) {
+    gk = c.g[k];
+    colk = __shfl_sync(kAll, col, 0);
+    for (int j = 0; j < k; ++j) {
+      const double nxt = __shfl_sync(kAll, col, j + 1);
+      const double cj = __shfl_sync(kAll, cs, j), sj = __shfl_sync(kAll, sn, j);
+      const double t = fma(cj, colk, sj * nxt);
+      colk = fma(cj, nxt, -sj * colk);
+      if (l == j) mine = t;
+    }
+    if (l < k) c.H[(size_t)k * ld + l] = mine;
+  } else if (w == 2) {
+    orth = c.orth;
+    wn2 = c.wn2;
+    orth1 = c.orth1;
+    const double t = (l < nk) ? hc[l] : 0.0;     // |h1|^2 = |w|^2 - |u|^2 (UPD_FIRST)
+    proj = warp_sum(t * t);
+  }
+  __syncthreads();
+  const double hn2 = S.hn2;
+  double rho = 0.0, hk1 = 0.0, csk = 1.0, snk = 0.0, inv_h = 0.0;
+  if (w == 2) {
+    const double grow = sqrt((double)nk) * orth;
+    double est = 0.0, r2 = 0.0;
+    if (phase == UPD_FIRST) {
+      r2 = (hn2 > 0.0) ? sqrt(hn2 / (hn2 + proj)) : 0.0;
+      est = (grow + 4.0 * nk * kEps) / r2;
+    } else {
+      // after the second pass: what is left of the first pass' loss orth1 is scaled by
+      // the basis' own loss, plus rounding, relative to the new norm
+      r2 = (wn2 > 0.0 && hn2 > 0.0) ? sqrt(hn2 / wn2) : 0.0;
+      if (r2 > 0.0) est = (grow * orth1 + 4.0 * nk * kEps) / r2;
+    }
+    if (l == 0) {
+      S.est = est;
+      S.rho2 = r2;
+    }
+  } else if (w == 1) {
+    hk1 = sqrt(hn2);
+    rho = hypot(colk, hk1);
+    // lanes 0, 1, 2: cos = colk / rho, sin = h_{k+1,k} / rho, 1 / h_{k+1,k}
+    const double num = (l == 0) ? colk : ((l == 1) ? hk1 : 1.0);
+    const double den = (l == 2) ? hk1 : rho;
+    const double q = (den > 0.0) ? num / den : ((l == 0) ? 1.0 : 0.0);
+    csk = __shfl_sync(kAll, q, 0);
+    snk = __shfl_sync(kAll, q, 1);
+    inv_h = __shfl_sync(kAll, q, 2);
+  }
+  __syncthreads();
+  if (w != 1) return;
+  if (phase == UPD_FIRST && hn2 > 0.0 && !(S.est <= kOrthTol)) {
+    if (l == 0) {
       c.reorth = 1;
       c.reorth_mask |= 1u << k;
-      c.orth1 = est;
+      c.orth1 = S.est;
       c.wn2 = hn2;
-      __threadfence();
-    } else {
-      if (hn2 > 0.0) c.orth = est;
-      givens_column<kL2>(c, b, hn2, hc, nullptr, k, restart, host_flags);
     }
-  } else {
-    // after the second pass: what is left of the first pass' loss orth1 is scaled by
-    // the basis' own loss, plus rounding, relative to the new norm
-    const double rho2 = (c.wn2 > 0.0 && hn2 > 0.0) ? sqrt(hn2 / c.wn2) : 0.0;
-    if (rho2 > 0.0) c.orth = fmax(c.orth, (grow * c.orth1 + 4.0 * nk * kEps) / rho2);
-    c.reorth = 0;
-    givens_column<kL2>(c, b, hn2, h1, hc, k, restart, host_flags);
+    return;
   }
+  const double gk1 = -snk * gk, gk0 = csk * gk;
+  const double res = fabs(gk1);
+  const bool stop = !(res > c.tol_abs) || (k + 1 >= restart) || !(hk1 > 0.0) ||
+                    !(rho > 0.0) || !isfinite(res);
+  if (l == 0) {
+    if (phase == UPD_FIRST) {
+      if (hn2 > 0.0) c.orth = S.est;
+    } else {
+      if (S.rho2 > 0.0) c.orth = fmax(c.orth, S.est);
+      c.reorth = 0;
+    }
+    c.H[(size_t)k * ld + k] = rho;
+    c.H[(size_t)k * ld + k + 1] = 0.0;
+    c.cs[k] = csk;
+    c.sn[k] = snk;
+    c.g[k] = gk0;
+    c.g[k + 1] = gk1;
+    c.res_est = res;
+    c.k_done = k + 1;
+    c.gmres_iters += 1;
+    c.inv_h = inv_h;
+    c.s[k + 1] = inv_h;
+    if (stop) c.gm_active = 0;
+    if (host_flag) *host_flag = stop ? 0 : 1;
+  }
+  if (!stop) return;
+  // y = R^-1 g: back substitution of the rotated Hessenberg matrix, lane j holding column
+  // j's entry of the current row (the next row's is loaded ahead)
+  __syncwarp();
+  const double g = (l == k) ? gk0 : ((l < k) ? c.g[l] : 0.0);
+  double row = (l == k) ? rho : 0.0, yj = 0.0;
+  for (int i = k; i >= 0; --i) {
+    const double next = (i > 0 && l >= i - 1 && l <= k) ? c.H[(size_t)l * ld + i - 1] : 0.0;
+    double s = __shfl_sync(kAll, g, i);
+    for (int j = i + 1; j <= k; ++j)
+      s = fma(-__shfl_sync(kAll, row, j), __shfl_sync(kAll, yj, j), s);
+    const double d = __shfl_sync(kAll, row, i);
+    if (l == i) yj = (d != 0.0) ? s / d : 0.0;
+    row = next;
+  }
+  if (l <= k) c.y[l] = yj;
 }
 
-// y = R^-1 g: back substitution of the rotated Hessenberg matrix of the finished cycle.
-// One thread.
-__device__ __forceinline__ void lsq_solve(VecCtl& c) {
-  const int kd = c.k_done;
-  const int ld = MCA_KMAX + 1;
-  for (int i = kd - 1; i >= 0; --i) {
-    double s = c.g[i];
-    for (int j = i + 1; j < kd; ++j) s -= c.H[(size_t)j * ld + i] * c.y[j];
-    const double d = c.H[(size_t)i * ld + i];
-    c.y[i] = (d != 0.0) ? s / d : 0.0;
+// Fixed-order reduction of part[b][j][0..nblk) into h_j = scale[j] * sum (j < nk) of vector
+// b, with scale[j] h_j behind it (kHStride), by the whole block of 256 threads (warp w takes
+// rows w, w + 8, ...).
+__device__ __forceinline__ void reduce_rows(const double* __restrict__ part, int b, int nblk,
+                                            int nk, double* __restrict__ h,
+                                            const double* scale) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  for (int j = w; j < nk; j += 8) {
+    double s = 0.0;
+    for (int t = l; t < nblk; t += 32) s += __ldcg(&part[((size_t)b * 32 + j) * nblk + t]);
+    s = warp_sum(s);
+    if (l == 0) {
+      const double v = s * scale[j];
+      h[(size_t)b * kHStride + j] = v;
+      h[(size_t)b * kHStride + 32 + j] = v * scale[j];
+    }
   }
 }
 

@@ -1,0 +1,79 @@
+"""The Krylov vector kernels at the sizes where their pairs of entries, half-block sums and
+per-length instantiations can go wrong: odd and even rows and columns, a pair across a row
+and across the two layers, one, two and three entries per accumulator, one to 30 basis
+vectors, buffers off the 16-byte boundary."""
+import numpy as np
+import pytest
+
+import mca_inputs as mi
+from oracle import mca_oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2109_07929_gb300 as mca  # noqa: E402
+
+DEV = "cuda:0"
+
+
+def _off(shape, off, dtype=torch.float64):
+    """A contiguous tensor whose data starts `off` entries into its allocation."""
+    n = int(np.prod(shape))
+    return torch.empty(n + 2, dtype=dtype, device=DEV)[off:off + n].view(shape)
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("m,n", [(1, 2), (3, 5), (5, 4), (2, 256), (31, 130), (33, 47),
+                                 (700, 300), (3, 1025)])
+def test_apply_does_not_depend_on_alignment(m, n, off):
+    """w = J z of the paired kernel (even n, 16-byte boundaries) and of the single-cell one:
+    the same operations per cell, so the same bits; against the oracle's FP64 product within
+    1e-14 of 8 |z|_max (the bound of the FP64 apply)."""
+    cb = mi.make_crossbar(m, n, 3, nvec=2)
+    rng = np.random.default_rng(m * n)
+    D = np.abs(rng.standard_normal((2, m * n))) * 1e-5
+    z = rng.standard_normal((2, 2 * m * n))
+    p = cb.params
+    with mca.Solver(mca.default_params(m, n, max_batch=2, flags=0), cb.gmap) as s:
+        Dd, zd, w = _off(D.shape, off), _off(z.shape, off), _off(z.shape, off)
+        Dd.copy_(torch.as_tensor(D))
+        zd.copy_(torch.as_tensor(z))
+        s.jacobian_apply(Dd, zd, w)
+        z32, w32 = _off(z.shape, off, torch.float32), _off(z.shape, off)
+        z32.copy_(zd.float())
+        s.jacobian_apply_f32(Dd, z32, w32)
+        ref, ref32 = _off(z.shape, 1), _off(z.shape, 1)
+        s.jacobian_apply(Dd, zd, ref)
+        s.jacobian_apply_f32(Dd, z32, ref32)
+    assert torch.equal(w, ref) and torch.equal(w32, ref32)
+    zero = np.zeros(m * n)
+    for v in range(2):
+        J = O.jacobian(p, D[v].reshape(m, n), zero, zero)
+        assert np.abs(w[v].cpu().numpy() - J @ z[v]).max() <= 1e-14 * 8 * np.abs(z[v]).max()
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("m,n,nvec", [(1, 3, 1), (5, 7, 2), (16, 130, 3), (64, 64, 1),
+                                      (640, 255, 1), (300, 512, 2), (768, 700, 1)])
+def test_gmres_reaches_its_tolerance(m, n, nvec, off):
+    """Restarted GMRES on J dx = rhs with the Jacobi preconditioner (long cycles, all basis
+    lengths; dx on and off a 16-byte boundary): the cycle's own residual estimate equals the
+    true residual of dx to 1e-6 (CGS with selective reorthogonalisation keeps the estimate
+    exact to about 30 * 1e-8)."""
+    cb = mi.make_crossbar(m, n, 5, nvec=nvec, gdist="uniform_paper", g_src=1.0,
+                          g_term_top_right=1.0, g_term_bot_top=1.0, g_sense=1.0, b=0.0)
+    p = cb.params
+    prm = mca.default_params(m, n, g_src=1.0, g_term_top_right=1.0, g_term_bot_top=1.0,
+                             g_sense=1.0, b=0.0, precision=mca.PREC_JACOBI, max_batch=nvec)
+    D = np.tile(cb.gmap.reshape(1, -1), (nvec, 1))
+    rhs = np.random.default_rng(7).standard_normal((nvec, 2 * m * n))
+    with mca.Solver(prm, cb.gmap) as s:
+        dx = _off(rhs.shape, off)
+        Dd, rd = torch.as_tensor(D, device=DEV), torch.as_tensor(rhs, device=DEV)
+        its, est = s.gmres_solve(Dd, D.mean(axis=1), rd, dx, 1e-9)
+    x = dx.cpu().numpy()
+    zero = np.zeros(m * n)
+    for v in range(nvec):
+        r = np.linalg.norm(rhs[v] - O.jacobian(p, cb.gmap, zero, zero) @ x[v])
+        scale = np.linalg.norm(rhs[v])
+        assert its[v] >= 1 and abs(r - est[v]) <= 1e-6 * r + 1e-13 * scale
