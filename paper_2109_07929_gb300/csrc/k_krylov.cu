@@ -81,15 +81,15 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
 // last block into h2_j = s_j <V_j, u>.  Rarely does any work, so a launch has a quarter of
 // the summation's blocks, each taking them in turn.
 // ZS: the Newton step from V = 0, whose v_0 is stored in the first column of the top layer
-// only (the residual's sparse_f); its other entries are not read.
+// only (the residual's sparse_f); its other entries are not read, and the last block also
+// subtracts h2_0 v_0 from u (see subtract_sparse_v0), in place of the update pass.
 template <int KP, bool ZS = false>
 __global__ void __launch_bounds__(kThreads)
-k_reorth_dots(const double* __restrict__ u, const double* __restrict__ V, size_t vstride,
-              size_t n2, int nk, double* __restrict__ part, int nblk,
+k_reorth_dots(double* u, const double* __restrict__ V, size_t vstride, size_t n2, int nk, double* __restrict__ part, int nblk,
               const VecCtl* __restrict__ ctl, unsigned int* cnt, double* h2, int ncols) {
   const int b = blockIdx.y;
   if (!ctl[b].gm_active || !ctl[b].reorth) return;
-  const double* ub = u + (size_t)b * vstride;
+  double* ub = u + (size_t)b * vstride;
   const double* Vb = V + (size_t)b * vstride;
   const int N2 = (int)n2;
   const int mn = N2 / 2, n = ncols;
@@ -110,26 +110,59 @@ k_reorth_dots(const double* __restrict__ u, const double* __restrict__ V, size_t
   if (last_block(cnt, b)) {
     reduce_rows(part, b, nblk, nk, h2, ctl[b].s);
     if (threadIdx.x == 0) cnt[b] = 0;
+    if (ZS) subtract_sparse_v0(ub, Vb, h2 + (size_t)b * kHStride, mn, n);
   }
 }
 
-// Passes 2 and 4: out <- w - sum_j hc_j v_j (the next, unnormalised basis vector, with
-// its BF16 copy for the tensor-core preconditioner), then the partial ||out||^2; the last
-// block of each vector runs the phase's control step (UpdPhase).
+// Passes 2 and 4: out <- w - sum_j hc_j v_j over j = j0 .. nk - 1 (the next, unnormalised
+// basis vector, with its BF16 copy for the tensor-core preconditioner), then the partial
+// ||out||^2; the last block of each vector runs the phase's control step (UpdPhase).  j0 = 1
+// in the Newton step from V = 0, where the dots' last block has subtracted the sparse v_0.
 //
-// Bound: the FP64 pipe from nk = 3 on (nk + 1 FMAs per entry), HBM below.  Entries go in
+// Bound: the FP64 pipe from three vectors on, HBM below.  A predicated-off FMA takes its
+// turn on that pipe like any other, so the number of vectors NK is exact: 1 .. 8, or any
+// (NK = 0) in groups of four and a rest by cases (at 1024 x 1024, 16 vectors, three of
+// them took as long as four, 312 us; now 239).  Entries go in
 // pairs (16-byte loads; n2 is even, so every vector starts on a 16-byte boundary): half a
 // block takes one block of the summation, two accumulators per thread.  Two pairs are in
-// flight per thread, all their loads issued before the first store (out may alias w): G = 1
-// the next trip of the same accumulators, G = 2 (when the accumulators have one trip or
-// two) another block of the summation.  With one entry per thread and a butterfly per warp
-// the reduction and the coefficients took more FP64 instructions than the update itself
-// (256 x 256, 8 vectors, nk = 1 and 2: 34 and 38 us, now 16 and 20).
+// flight per thread, all their loads issued before the first store (out may alias w, so the
+// compiler cannot move loads of the next trip above the stores): G = 1 the next trip of the
+// same accumulators, G = 2 (when the accumulators have one trip or two) another block of
+// the summation.  With one entry per thread and a butterfly per warp the reduction and the
+// coefficients took more FP64 instructions than the update itself (256 x 256, 8 vectors,
+// nk = 1 and 2: 34 and 38 us, now 16 and 20).
 // (layer, i, j) of a pair comes from one multiply-and-shift quotient.
-template <int KP, bool ZS, int G>
-__global__ void __launch_bounds__(kThreads, KP <= 4 ? 4 : (KP <= 8 ? 3 : 2))
+template <int N>
+__device__ __forceinline__ void subtract(const double* __restrict__ v, size_t n2,
+                                         const double* hj, uint32_t p, double2& x) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const double2 t = reinterpret_cast<const double2*>(v + (size_t)j * n2)[p];
+    x.x = fma(-hj[j], t.x, x.x);
+    x.y = fma(-hj[j], t.y, x.y);
+  }
+}
+
+// the same for two pairs, with both pairs' loads of a vector together
+template <int N>
+__device__ __forceinline__ void subtract2(const double* __restrict__ v, size_t n2,
+                                          const double* hj, uint32_t p, uint32_t q, double2& x,
+                                          double2& y) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const double2* vj = reinterpret_cast<const double2*>(v + (size_t)j * n2);
+    const double2 t = vj[p], u = vj[q];
+    x.x = fma(-hj[j], t.x, x.x);
+    x.y = fma(-hj[j], t.y, x.y);
+    y.x = fma(-hj[j], u.x, y.x);
+    y.y = fma(-hj[j], u.y, y.y);
+  }
+}
+
+template <int NK, int G>
+__global__ void __launch_bounds__(kThreads, NK <= 4 ? 4 : 3)
 k_update_norm(int phase, const double* w, size_t wstride, const double* __restrict__ V,
-              size_t vstride, size_t n2, int nk, const double* __restrict__ hc,
+              size_t vstride, size_t n2, int nk, int j0, const double* __restrict__ hc,
               double* __restrict__ part, int nblk, VecCtl* ctl, unsigned int* cnt,
               const double* __restrict__ h1, int restart, int32_t* host_flags, double* out,
               size_t ostride, __nv_bfloat16* __restrict__ xbf, int mp, int np, int m, int n,
@@ -137,13 +170,19 @@ k_update_norm(int phase, const double* w, size_t wstride, const double* __restri
   const int b = blockIdx.y;
   if (phase != UPD_PLAIN && (!ctl[b].gm_active || (phase == UPD_REORTH && !ctl[b].reorth)))
     return;
-  double hj[KP];
+  const double* hs = hc + (size_t)b * kHStride + 32 + j0;      // their scaled coefficients
+  double hj[NK > 0 ? NK : 1];
+  __shared__ double hsh[32];
+  if constexpr (NK > 0) {
 #pragma unroll
-  for (int j = 0; j < KP; ++j)
-    hj[j] = (j < nk) ? hc[(size_t)b * kHStride + 32 + j] : 0.0;
+    for (int j = 0; j < NK; ++j) hj[j] = hs[j];
+  } else {
+    if ((int)threadIdx.x < nk - j0) hsh[threadIdx.x] = hs[threadIdx.x];
+    __syncthreads();
+  }
   const double2* wb = reinterpret_cast<const double2*>(w + (size_t)b * wstride);
   double2* ob = reinterpret_cast<double2*>(out + (size_t)b * ostride);
-  const double* Vb = V + (size_t)b * vstride;
+  const double* Vb = V + (size_t)b * vstride + (size_t)j0 * n2;
   __nv_bfloat16* xb = xbf ? xbf + (size_t)b * 2 * mp * np : nullptr;
   const uint32_t mn = (uint32_t)(n2 / 2), P = mn;      // P pairs = m n
   const bool even = (n & 1) == 0;                      // no pair crosses a row
@@ -171,36 +210,30 @@ k_update_norm(int phase, const double* w, size_t wstride, const double* __restri
     acc[0] = fma(x.x, x.x, acc[0]);
     acc[1] = fma(x.y, x.y, acc[1]);
   };
-  // x -= hj_j V_j of pair p.  ZS: v_0 is stored (and nonzero) in the first column of the
-  // top layer only
-  auto sub = [&](int j, uint32_t p, double2& x) {
-    const double* vj = Vb + (size_t)j * n2;
-    if (ZS && j == 0) {
-      const uint32_t e = 2 * p;
-      if (e < mn && by_n.quot(e) * (uint32_t)n == e) x.x = fma(-hj[0], vj[e], x.x);
-      if (e + 1 < mn && by_n.quot(e + 1) * (uint32_t)n == e + 1)
-        x.y = fma(-hj[0], vj[e + 1], x.y);
-    } else {
-      const double2 v = reinterpret_cast<const double2*>(vj)[p];
-      x.x = fma(-hj[j], v.x, x.x);
-      x.y = fma(-hj[j], v.y, x.y);
-    }
-  };
   auto one = [&](uint32_t p, double (&acc)[2]) {
     double2 x = wb[p];
-#pragma unroll
-    for (int j = 0; j < KP; ++j)
-      if (j < nk) sub(j, p, x);
+    if constexpr (NK > 0) {
+      subtract<NK>(Vb, n2, hj, p, x);
+    } else {
+      for (int j = 0; j < nk - j0; ++j) subtract<1>(Vb + (size_t)j * n2, n2, hsh + j, p, x);
+    }
     finish(p, x, acc);
   };
   auto two = [&](uint32_t p, uint32_t q, double (&accp)[2], double (&accq)[2]) {
     double2 x = wb[p], y = wb[q];
-#pragma unroll
-    for (int j = 0; j < KP; ++j)
-      if (j < nk) {
-        sub(j, p, x);
-        sub(j, q, y);
+    if constexpr (NK > 0) {
+      subtract2<NK>(Vb, n2, hj, p, q, x, y);
+    } else {
+      int j = 0;
+      const double* vj = Vb;
+      for (; j + 4 <= nk - j0; j += 4, vj += 4 * n2) subtract2<4>(vj, n2, hsh + j, p, q, x, y);
+      switch (nk - j0 - j) {
+        case 1: subtract2<1>(vj, n2, hsh + j, p, q, x, y); break;
+        case 2: subtract2<2>(vj, n2, hsh + j, p, q, x, y); break;
+        case 3: subtract2<3>(vj, n2, hsh + j, p, q, x, y); break;
+        default: break;
       }
+    }
     finish(p, x, accp);
     finish(q, y, accq);
   };
@@ -427,17 +460,7 @@ void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
   k_reduce_dots<<<B, kThreads, 0, s>>>(part, nblk, nk, h, ctl);
 }
 
-#define MCA_KP_DISPATCH(nk, CALL)      \
-  do {                                 \
-    if ((nk) <= 1) CALL(1);            \
-    else if ((nk) <= 2) CALL(2);       \
-    else if ((nk) <= 4) CALL(4);       \
-    else if ((nk) <= 8) CALL(8);       \
-    else if ((nk) <= 16) CALL(16);     \
-    else CALL(32);                     \
-  } while (0)
-
-void launch_reorth_dots(const double* u, const double* V, size_t vstride, size_t n2, int nk,
+void launch_reorth_dots(double* u, const double* V, size_t vstride, size_t n2, int nk,
                         double* part, int nblk, int B, const VecCtl* ctl, unsigned int* cnt,
                         double* h2, cudaStream_t s, bool zs, int ncols) {
   const dim3 grid((nblk + 3) / 4, B);
@@ -450,7 +473,11 @@ void launch_reorth_dots(const double* u, const double* V, size_t vstride, size_t
       k_reorth_dots<KP_, false><<<grid, kThreads, 0, s>>>(u, V, vstride, n2, nk, part, nblk, \
                                                           ctl, cnt, h2, ncols);              \
   } while (0)
-  MCA_KP_DISPATCH(nk, MCA_CALL);
+  if (nk <= 2) MCA_CALL(2);
+  else if (nk <= 4) MCA_CALL(4);
+  else if (nk <= 8) MCA_CALL(8);
+  else if (nk <= 16) MCA_CALL(16);
+  else MCA_CALL(32);
 #undef MCA_CALL
 }
 
@@ -465,20 +492,30 @@ void launch_update_norm(int phase, const double* w, size_t wstride, const double
   const bool four = n2 <= 2 * (size_t)nblk * kThreads;
   const dim3 grid(four ? (nblk + 3) / 4 : (nblk + 1) / 2, B);
   const FastDiv by_n(n);
-#define MCA_CALL3(KP_, ZS_, G_)                                                             \
-  k_update_norm<KP_, ZS_, G_><<<grid, kThreads, 0, s>>>(                                    \
-      phase, w, wstride, V, vstride, n2, nk, hc, part, nblk, ctl, cnt, h1, restart,         \
-      host_flags, out, ostride, xbf, mp, np, m, n, by_n)
-#define MCA_CALL(KP_)                                                                       \
+  const int j0 = zs ? 1 : 0;
+#define MCA_CALL(NK_)                                                                       \
   do {                                                                                      \
-    if (zs && four) MCA_CALL3(KP_, true, 2);                                                \
-    else if (zs) MCA_CALL3(KP_, true, 1);                                                   \
-    else if (four) MCA_CALL3(KP_, false, 2);                                                \
-    else MCA_CALL3(KP_, false, 1);                                                          \
+    if (four)                                                                               \
+      k_update_norm<NK_, 2><<<grid, kThreads, 0, s>>>(                                      \
+          phase, w, wstride, V, vstride, n2, nk, j0, hc, part, nblk, ctl, cnt, h1, restart, \
+          host_flags, out, ostride, xbf, mp, np, m, n, by_n);                               \
+    else                                                                                    \
+      k_update_norm<NK_, 1><<<grid, kThreads, 0, s>>>(                                      \
+          phase, w, wstride, V, vstride, n2, nk, j0, hc, part, nblk, ctl, cnt, h1, restart, \
+          host_flags, out, ostride, xbf, mp, np, m, n, by_n);                               \
   } while (0)
-  MCA_KP_DISPATCH(nk, MCA_CALL);
+  switch (nk - j0) {
+    case 1: MCA_CALL(1); break;
+    case 2: MCA_CALL(2); break;
+    case 3: MCA_CALL(3); break;
+    case 4: MCA_CALL(4); break;
+    case 5: MCA_CALL(5); break;
+    case 6: MCA_CALL(6); break;
+    case 7: MCA_CALL(7); break;
+    case 8: MCA_CALL(8); break;
+    default: MCA_CALL(0); break;
+  }
 #undef MCA_CALL
-#undef MCA_CALL3
 }
 
 template <typename ZT>

@@ -34,6 +34,8 @@
 // stops taking items, frees its TMEM and returns.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "bits.cuh"
 #include "mca_internal.cuh"
 #include "solver_dev.cuh"
@@ -612,69 +614,75 @@ __device__ bool residual_phase(const PersistShape& sh, const double* gmap, const
   double sf = 0.0, sd = 0.0;
   float sdf = 0.f, sfh = 0.f, sfl = 0.f;
   bool dnot32 = false;
-  for (int base = threadIdx.x; base < mn; base += kUR * kPT) {
-    int iu[kUR], ju[kUR];
-    double vt[kUR], vb[kUR], tl[kUR], tr[kUR], bu[kUR], bd[kUR], g[kUR], vi[kUR];
+  // fast_c: a nonlinear device with norm32, chosen per phase (an FP64 instruction that a choice
+  // per cell predicates off still takes its turn on the FP64 pipe)
+  auto cells = [&](auto fast_c) {
+    constexpr bool kFast = decltype(fast_c)::value;
+    for (int base = threadIdx.x; base < mn; base += kUR * kPT) {
+      int iu[kUR], ju[kUR];
+      double vt[kUR], vb[kUR], tl[kUR], tr[kUR], bu[kUR], bd[kUR], g[kUR], vi[kUR];
 #pragma unroll
-    for (int u = 0; u < kUR; ++u) {
-      const int c = base + u * kPT;
-      const int cc = c < mn ? c : base;
-      iu[u] = cc / n;
-      ju[u] = cc - iu[u] * n;
-      g[u] = gmap[cc];
-      vi[u] = (ju[u] == 0) ? vin[iu[u]] : 0.0;
-      if (!ZERO) {
-        vt[u] = Vt[cc];
-        vb[u] = Vb[cc];
-        tl[u] = (ju[u] > 0) ? Vt[cc - 1] : 0.0;
-        tr[u] = (ju[u] < n - 1) ? Vt[cc + 1] : 0.0;
-        bu[u] = (iu[u] > 0) ? Vb[cc - n] : 0.0;
-        bd[u] = (iu[u] < m - 1) ? Vb[cc + n] : 0.0;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kUR; ++u) {
-      const int c = base + u * kPT;
-      if (c >= mn) break;
-      const int i = iu[u], j = ju[u];
-      double ft, fb, dg;
-      float dgf = 0.f;
-      if (ZERO) {
-        ft = (j == 0) ? -gr.g_src * vi[u] : 0.0;
-        fb = 0.0;
-        dg = g[u];
-        dgf = d2f_round(dg);
-      } else {
-        cell_residual_vals<YAK>(gr, i, j, vt[u], vb[u], tl[u], tr[u], bu[u], bd[u], g[u],
-                                vi[u], ft, fb, dg, dgf);
-      }
-      Ft[c] = ft;
-      Fb[c] = fb;
-      if (!ZERO) w.D[c] = dg;        // (the zero state's D is g: the apply reads the map)
-      {
-        const uint32_t dh = (uint32_t)__double2hiint(dg), dlw = (uint32_t)__double2loint(dg);
-        const uint32_t de = (dh >> 20) & 0x7FFu;
-        dnot32 |= ((dlw & 0x1FFFFFFFu) != 0u) ||
-                  (de - 897u > 253u && ((dh & 0x7FFFFFFFu) | dlw));
-      }
-      if (!ZERO || j == 0) {         // the zero state's F is zero off the first column, and
-        w.xbf[tix(i, j, 2 * mp)] = d2bf16_bits(ft);   // the BF16 copy starts zeroed
-        if (!ZERO) w.xbf[tix(mp + i, j, 2 * mp)] = d2bf16_bits(fb);
-      }
-      if (!ZERO) {
-        if (!norm32) {
-          sf = fma(ft, ft, sf);
-          sf = fma(fb, fb, sf);
-        } else {
-          const float a = d2f_round(ft), bb = d2f_round(fb);
-          float e;
-          sfh = two_sum(sfh, fmaf(a, a, bb * bb), e);
-          sfl += e;
+      for (int u = 0; u < kUR; ++u) {
+        const int c = base + u * kPT;
+        const int cc = c < mn ? c : base;
+        iu[u] = (int)sh.by_n.quot((uint32_t)cc);
+        ju[u] = cc - iu[u] * n;
+        g[u] = gmap[cc];
+        vi[u] = (ju[u] == 0) ? vin[iu[u]] : 0.0;
+        if (!ZERO) {
+          vt[u] = Vt[cc];
+          vb[u] = Vb[cc];
+          tl[u] = (ju[u] > 0) ? Vt[cc - 1] : 0.0;
+          tr[u] = (ju[u] < n - 1) ? Vt[cc + 1] : 0.0;
+          bu[u] = (iu[u] > 0) ? Vb[cc - n] : 0.0;
+          bd[u] = (iu[u] < m - 1) ? Vb[cc + n] : 0.0;
         }
       }
-      if (lin) sd += dg; else sdf += dgf;
+#pragma unroll
+      for (int u = 0; u < kUR; ++u) {
+        const int c = base + u * kPT;
+        if (c >= mn) break;
+        const int i = iu[u], j = ju[u];
+        double ft, fb, dg;
+        float dgf = 0.f;
+        if (ZERO) {
+          ft = (j == 0) ? -gr.g_src * vi[u] : 0.0;
+          fb = 0.0;
+          dg = g[u];
+          dgf = d2f_round(dg);
+        } else {
+          cell_residual_vals<YAK>(gr, i, j, vt[u], vb[u], tl[u], tr[u], bu[u], bd[u], g[u],
+                                  vi[u], ft, fb, dg, dgf);
+        }
+        Ft[c] = ft;
+        Fb[c] = fb;
+        if (!ZERO) w.D[c] = dg;      // (the zero state's D is g: the apply reads the map)
+        {
+          const uint32_t dh = (uint32_t)__double2hiint(dg), dlw = (uint32_t)__double2loint(dg);
+          const uint32_t de = (dh >> 20) & 0x7FFu;
+          dnot32 |= ((dlw & 0x1FFFFFFFu) != 0u) ||
+                    (de - 897u > 253u && ((dh & 0x7FFFFFFFu) | dlw));
+        }
+        if (!ZERO || j == 0) {       // the zero state's F is zero off the first column, and
+          w.xbf[tix(i, j, 2 * mp)] = d2bf16_bits(ft);   // the BF16 copy starts zeroed
+          if (!ZERO) w.xbf[tix(mp + i, j, 2 * mp)] = d2bf16_bits(fb);
+        }
+        if (!ZERO) {
+          if (kFast || norm32) {
+            const float a = d2f_round(ft), bb = d2f_round(fb);
+            float e;
+            sfh = two_sum(sfh, fmaf(a, a, bb * bb), e);
+            sfl += e;
+          } else {
+            sf = fma(ft, ft, sf);
+            sf = fma(fb, fb, sf);
+          }
+        }
+        if (!kFast && lin) sd += dg; else sdf += dgf;
+      }
     }
-  }
+  };
+  if (!lin && (ZERO || norm32)) cells(std::true_type{}); else cells(std::false_type{});
   sd += f2d_bits(sdf);
   sf += f2d_bits(sfh) + f2d_bits(sfl);
   const int any64 = __syncthreads_or(dnot32 ? 1 : 0);

@@ -14,6 +14,7 @@
 // instead of the FP64 library functions.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "bits.cuh"
 #include "mca_internal.cuh"
@@ -389,13 +390,30 @@ k_residual(Grid gr, const double* __restrict__ gmap, const double* __restrict__ 
   const bool lin = (gr.b == 0.0);
   double sf = 0.0, sd = 0.0;
   float sdf = 0.f, ss = 0.f;
-  auto emit = [&](int c, double ft, double fb, double dg, float dgf) {
+  // lin_c: the sums of a linear device, chosen per launch (see k_residual_newton)
+  auto emit = [&](auto lin_c, int c, double ft, double fb, double dg, float dgf) {
     Ft[c] = ft;
     Fb[c] = fb;
     Db[c] = dg;
     sf = fma(ft, ft, sf);
     sf = fma(fb, fb, sf);
-    if (lin) sd += dg; else sdf += dgf;
+    if constexpr (decltype(lin_c)::value) sd += dg; else sdf += dgf;
+  };
+  auto cells = [&](auto lin_c) {
+    for (int c = blockIdx.x * kThreads + threadIdx.x; c < mn; c += nblk * kThreads) {
+      const int i = c / n;
+      const int j = c - i * n;
+      double ft, fb, dg;
+      float dgf;
+      [[maybe_unused]] float f32a, f32b;
+      if constexpr (PAIR)
+        cell_residual_pair<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb,
+                                dg, dgf, ss, f32a, f32b);
+      else
+        cell_residual<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb, dg,
+                           dgf);
+      emit(lin_c, c, ft, fb, dg, dgf);
+    }
   };
   bool walked = false;
   if constexpr (PAIR) {
@@ -407,26 +425,13 @@ k_residual(Grid gr, const double* __restrict__ gmap, const double* __restrict__ 
                         cell_residual_pair_split<YAK>(gr, i, j, vt, vb, tl, tr, bu, bd, gmap[c],
                                                       (j == 0) ? vinb[i] : 0.0, ft, fb, dg,
                                                       dgf, ss, f32a, f32b);
-                        emit(c, ft, fb, dg, dgf);
+                        emit(std::false_type{}, c, ft, fb, dg, dgf);
                       });
       walked = true;
     }
   }
   if (!walked) {
-    for (int c = blockIdx.x * kThreads + threadIdx.x; c < mn; c += nblk * kThreads) {
-      const int i = c / n;
-      const int j = c - i * n;
-      double ft, fb, dg;
-      float dgf;
-      float f32a, f32b;
-      if constexpr (PAIR)
-        cell_residual_pair<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb,
-                                dg, dgf, ss, f32a, f32b);
-      else
-        cell_residual<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb, dg,
-                           dgf);
-      emit(c, ft, fb, dg, dgf);
-    }
+    if (!PAIR && lin) cells(std::true_type{}); else cells(std::false_type{});
   }
   sd += f2d_bits(sdf);
   constexpr int kRows = PAIR ? 3 : 2;
@@ -491,11 +496,15 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
   double sf = 0.0, sd = 0.0;
   float sdf = 0.f, ss = 0.f, sfh = 0.f, sfl = 0.f;
   bool dnot32 = false;
-  // grid-stride walk over the cells with (i, j) advanced incrementally (no division per
-  // cell); the BF16 copy sits in the padded [layer][mp][np] layout at row offset i * np
-  // the stores and sums of one cell (both cell forms and both walks)
-  auto emit = [&](int i, int j, int c, double ft, double fb, double dg, float dgf, float ft32,
-                  float fb32) {
+  // The stores and sums of one cell (both cell forms and both walks); the BF16 copy sits in
+  // the padded [layer][mp][np] layout at row offset i * np.  pair_c: the pair cell.  fast_c:
+  // the sums a nonlinear device with norm32 takes, chosen per launch and not per cell: an FP64
+  // instruction that a run-time choice predicates off still takes its turn on the FP64 pipe
+  // (18.3 per cell were issued for the 10 of the cell; 1024 x 1024, 16 vectors: 556 us, now
+  // 402).
+  auto emit = [&](auto fast_c, auto pair_c, int i, int j, int c, double ft, double fb,
+                  double dg, float dgf, float ft32, float fb32) {
+    constexpr bool kFast = decltype(fast_c)::value, kPair = decltype(pair_c)::value;
     if (!sparse_f || j == 0) Ft[c] = ft;
     if (!sparse_f) Fb[c] = fb;
     Db[c] = dg;
@@ -508,7 +517,7 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
     }
     if (xt != nullptr) {
       const int o = i * np + j;
-      if (PAIR && use_pair) {
+      if constexpr (kPair) {
         xt[o] = f2bf16_bits(ft32);
         xt[o + mp * np] = f2bf16_bits(fb32);
       } else {
@@ -516,36 +525,29 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
         xt[o + mp * np] = d2bf16_bits(fb);
       }
     }
-    if (!ZERO) {
-      if ((PAIR && use_pair) || !norm32) {
+    if constexpr (!ZERO) {
+      if constexpr (kPair) {
         sf = fma(ft, ft, sf);
         sf = fma(fb, fb, sf);
-      } else {
+      } else if (kFast || norm32) {
         const float a = d2f_round(ft), bb = d2f_round(fb);
         float e;
         sfh = two_sum(sfh, fmaf(a, a, bb * bb), e);
         sfl += e;
+      } else {
+        sf = fma(ft, ft, sf);
+        sf = fma(fb, fb, sf);
       }
     }
-    if (lin) sd += dg; else sdf += dgf;
-  };
-  bool walked = false;
-  if constexpr (PAIR && !ZERO) {
-    // pair cells of a grid whose columns fill the strips: split each voltage once
-    if (use_pair && strip_walk_fits(n)) {
-      pair_strip_walk(m, n, Vt, Vb, nblk,
-                      [&](int i, int j, int c, F2 vt, F2 vb, F2 tl, F2 tr, F2 bu, F2 bd) {
-                        double ft, fb, dg;
-                        float dgf, ft32, fb32;
-                        cell_residual_pair_split<YAK>(gr, i, j, vt, vb, tl, tr, bu, bd, gmap[c],
-                                                      (j == 0) ? vinb[i] : 0.0, ft, fb, dg,
-                                                      dgf, ss, ft32, fb32);
-                        emit(i, j, c, ft, fb, dg, dgf, ft32, fb32);
-                      });
-      walked = true;
+    if constexpr (kFast || kPair) {
+      sdf += dgf;
+    } else {
+      if (lin) sd += dg; else sdf += dgf;
     }
-  }
-  if (!walked) {
+  };
+  // grid-stride walk over the cells with (i, j) advanced incrementally (no division per
+  // cell)
+  auto cells = [&](auto fast_c, auto pair_c) {
     const int S = nblk * kThreads;
     const int Si = S / n, Sj = S - Si * n;
     int c = blockIdx.x * kThreads + threadIdx.x;
@@ -553,19 +555,19 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
     for (; c < mn; c += S) {
       double ft, fb, dg;
       float dgf = 0.f, ft32 = 0.f, fb32 = 0.f;
-      if (ZERO) {
+      if constexpr (ZERO) {
         ft = (j == 0) ? -gr.g_src * vinb[i] : 0.0;
         fb = 0.0;
         dg = gmap[c];
         dgf = d2f_round(dg);
-      } else if (PAIR && use_pair) {
+      } else if constexpr (decltype(pair_c)::value) {
         cell_residual_pair<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb,
                                 dg, dgf, ss, ft32, fb32);
       } else {
         cell_residual<YAK>(gr, i, j, c, Vt, Vb, gmap[c], (j == 0) ? vinb[i] : 0.0, ft, fb, dg,
                            dgf);
       }
-      emit(i, j, c, ft, fb, dg, dgf, ft32, fb32);
+      emit(fast_c, pair_c, i, j, c, ft, fb, dg, dgf, ft32, fb32);
       j += Sj;
       i += Si;
       if (j >= n) {
@@ -573,6 +575,30 @@ k_residual_newton(Grid gr, const double* __restrict__ gmaps, const int* __restri
         ++i;
       }
     }
+  };
+  constexpr std::true_type yes{};
+  constexpr std::false_type no{};
+  if (PAIR && !ZERO && use_pair) {
+    // (the pair cell's device is nonlinear)  a grid whose columns fill the strips: split
+    // each voltage once
+    if constexpr (PAIR && !ZERO) {
+      if (strip_walk_fits(n))
+        pair_strip_walk(m, n, Vt, Vb, nblk,
+                        [&](int i, int j, int c, F2 vt, F2 vb, F2 tl, F2 tr, F2 bu, F2 bd) {
+                          double ft, fb, dg;
+                          float dgf, ft32, fb32;
+                          cell_residual_pair_split<YAK>(gr, i, j, vt, vb, tl, tr, bu, bd,
+                                                        gmap[c], (j == 0) ? vinb[i] : 0.0, ft,
+                                                        fb, dg, dgf, ss, ft32, fb32);
+                          emit(yes, yes, i, j, c, ft, fb, dg, dgf, ft32, fb32);
+                        });
+      else
+        cells(yes, yes);
+    }
+  } else if (!lin && (ZERO || norm32)) {
+    cells(yes, no);
+  } else {
+    cells(no, no);
   }
   sd += f2d_bits(sdf);
   sf += f2d_bits(sfh) + f2d_bits(sfl);
@@ -732,6 +758,8 @@ __device__ __forceinline__ int half_scatter_index(int lane) {
 // Bound: the FP64 pipe from nk = 2 on (2 nk FMAs per cell and the apply's own instructions),
 // HBM below.  1024 x 1024, 16 vectors, nk = 1: 170 us one cell per thread, 157 us in pairs;
 // 256 x 256, 8 vectors, first step: 13.0 and 8.7 us.
+// KP >= nk accumulators; exact up to nk = 8, because an FMA predicated off still takes its
+// turn on the FP64 pipe (1024 x 1024, 16 vectors, nk = 3: 329 us with four, 264 with three).
 template <int KP, typename ZT, int AM, bool ZS, int W>
 __global__ void __launch_bounds__(kThreads)
 k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
@@ -750,7 +778,8 @@ k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
   double* wt = w + (size_t)b * n2;
   double* wb = wt + mn;
   const double* Vb_ = V + (size_t)b * vstride;
-  double acc[W][KP] = {};
+  constexpr int KPP = KP <= 1 ? 1 : (KP <= 2 ? 2 : (KP <= 4 ? 4 : (KP <= 8 ? 8 : (KP <= 16 ? 16 : 32))));
+  double acc[W][KPP] = {};
   const int half = (W == 2) ? (int)threadIdx.x / (kThreads / 2) : 0;
   const int vb = W * blockIdx.x + half;                 // block of the summation
   const int lane_c = (W == 2) ? 2 * ((int)threadIdx.x & (kThreads / 2 - 1)) : (int)threadIdx.x;
@@ -815,15 +844,15 @@ k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
     }
   }
   if (V == nullptr) return;
-  __shared__ double red[W][kThreads / 32][KP];
+  __shared__ double red[W][kThreads / 32][KPP];
   const int wv = threadIdx.x >> 5, l = threadIdx.x & 31;
   if constexpr (W == 2) {
-    const double tot = half_sum_scatter<KP>(acc);
-    if ((l & (16 / KP - 1)) == 0)
-      red[half][(wv & 3) * 2 + (l >> 4)][half_scatter_index<KP>(l)] = tot;
+    const double tot = half_sum_scatter<KPP>(acc);
+    if ((l & (16 / KPP - 1)) == 0)
+      red[half][(wv & 3) * 2 + (l >> 4)][half_scatter_index<KPP>(l)] = tot;
   } else {
-    const double tot = warp_sum_scatter<KP>(acc[0]);
-    if (warp_scatter_writer<KP>(l)) red[0][wv][warp_scatter_index<KP>(l)] = tot;
+    const double tot = warp_sum_scatter<KPP>(acc[0]);
+    if (warp_scatter_writer<KPP>(l)) red[0][wv][warp_scatter_index<KPP>(l)] = tot;
   }
   __syncthreads();
   if (threadIdx.x < W * KP) {
@@ -845,6 +874,7 @@ k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
   // the stored basis is unnormalised: <v_j, w> = s_j <V_j, w>
   reduce_rows(part, b, nblk, nk, h, ctl[b].s);
   if (threadIdx.x == 0) cnt[b] = 0;
+  if (ZS) subtract_sparse_v0(wt, Vb_, h + (size_t)b * kHStride, mn, n);
 }
 
 // Output currents and the Kirchhoff balance per vector.
@@ -950,16 +980,33 @@ void spmv_dots(const Grid& gr, const double* D, const ZT* z, size_t zstride, dou
   const bool two = (gr.n & 1) == 0 && on(D, 16) && on(w, 16) && on(V, 16) &&
                    on(z, 2 * sizeof(ZT)) && (zstride & 1) == 0 && (vstride & 1) == 0;
   const FastDiv by_n(gr.n);
+  // the arithmetics the solver runs with dots; the others only serve mca_jacobian_apply_f32
+  constexpr bool kDots = std::is_same<ZT, double>::value || AM == kApplyPair || ZS;
 #define MCA_SPMV1(KP_, W_)                                                                   \
   k_spmv_dots<KP_, ZT, AM, ZS, W_><<<dim3((nblk + W_ - 1) / W_, B), kThreads, 0, s>>>(       \
       gr, D, z, zstride, w, V, vstride, nk, part, nblk, ctl, cnt, h, by_n)
 #define MCA_SPMV(KP_) do { if (two) MCA_SPMV1(KP_, 2); else MCA_SPMV1(KP_, 1); } while (0)
-  if (nk <= 1) MCA_SPMV(1);
-  else if (nk <= 2) MCA_SPMV(2);
-  else if (nk <= 4) MCA_SPMV(4);
-  else if (nk <= 8) MCA_SPMV(8);
-  else if (nk <= 16) MCA_SPMV1(16, 1);
-  else MCA_SPMV1(32, 1);
+  if (V == nullptr) {
+    MCA_SPMV(1);
+  } else if constexpr (kDots) {
+    switch (nk) {
+      case 0: case 1: MCA_SPMV(1); break;
+      case 2: MCA_SPMV(2); break;
+      case 3: MCA_SPMV(3); break;
+      case 4: MCA_SPMV(4); break;
+      case 5: MCA_SPMV(5); break;
+      case 6: MCA_SPMV(6); break;
+      case 7: MCA_SPMV(7); break;
+      case 8: MCA_SPMV(8); break;
+      default:
+        if (nk <= 10) MCA_SPMV1(10, 1);
+        else if (nk <= 12) MCA_SPMV1(12, 1);
+        else if (nk <= 16) MCA_SPMV1(16, 1);
+        else if (nk <= 20) MCA_SPMV1(20, 1);
+        else if (nk <= 24) MCA_SPMV1(24, 1);
+        else MCA_SPMV1(32, 1);
+    }
+  }
 #undef MCA_SPMV
 #undef MCA_SPMV1
 }

@@ -1397,6 +1397,7 @@ int mca_batch_create(mca_handle* const* hs, int32_t nh, int32_t max_ctas, mca_ba
     PersistShape& ps = shp[k];
     ps.gr = h->gr;
     ps.cfg = make_cfg(h);
+    ps.by_n = FastDiv(h->n);
     ps.mp = h->mp;
     ps.np = h->np;
     ps.gmaps = h->g;

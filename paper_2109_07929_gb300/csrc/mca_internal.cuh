@@ -268,7 +268,7 @@ void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
                         const VecCtl* ctl, cudaStream_t s);
 // pass 2: w -= V h1, partial dots <V_j, w>; the last block reduces them into h2.
 // Update passes of the Gram-Schmidt step (phase of launch_update_norm):
-//   UPD_PLAIN  out = w - V hc and ||out||^2 partials only (cnt, ctl unused)
+//   UPD_PLAIN  out = w and ||out||^2 partials only (nk = 0; cnt, ctl unused)
 //   UPD_FIRST  out = w - V h1 (hc = h1); the last block of each vector estimates the loss
 //              of orthogonality of out and either finishes Hessenberg column nk-1 (Givens
 //              rotation, scale of the new basis vector, flags) or marks the vector for the
@@ -278,8 +278,10 @@ void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
 enum UpdPhase { UPD_PLAIN = 0, UPD_FIRST = 1, UPD_REORTH = 2 };
 // second-pass dots h2 = V^T u (j < nk) of the new vector u (u[b] at u + b*vstride), only
 // for the vectors marked by UPD_FIRST
-// zs: the Newton step from V = 0 with a sparse v_0 (see launch_residual_newton), ncols = n
-void launch_reorth_dots(const double* u, const double* V, size_t vstride, size_t n2, int nk,
+// zs: the Newton step from V = 0 with a sparse v_0 (see launch_residual_newton), ncols = n;
+// the dots' last block then also subtracts v_0's part, h_0 v_0, from the vector itself (here
+// u, in launch_spmv_dots w), and the update pass starts with v_1
+void launch_reorth_dots(double* u, const double* V, size_t vstride, size_t n2, int nk,
                         double* part, int nblk, int B, const VecCtl* ctl, unsigned int* cnt,
                         double* h2, cudaStream_t s, bool zs = false, int ncols = 1);
 // out[b] at out + b*ostride, w[b] at w + b*wstride; BF16 copy of out in xbf (may be NULL)
@@ -337,6 +339,7 @@ void launch_modes_2x2_f64(double* Xh, const double* mu, const double* nu, int m,
 struct PersistShape {
   Grid gr;
   SolverCfg cfg;
+  FastDiv by_n{1};                      // quotient by gr.n
   int mp, np;
   const double* gmaps;                  // n_maps * m*n
   const float* mu_f;                    // np

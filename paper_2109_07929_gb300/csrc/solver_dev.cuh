@@ -132,7 +132,7 @@ __device__ __forceinline__ void negative_bias(const Grid& gr, double dv, double&
 // Yakopcic-form device (a compile-time choice, so the sinh device pays nothing for it).
 // FP64 instructions: the device voltage 1, the current 3 (device_current), and per layer
 // the neighbour sum and two FMAs that add the wire diagonal term and the coupling term to
-// the current (10 in all; the source term adds one on the first column).
+// the current (10 in all).
 // The arithmetic of cell_residual on the cell's loaded voltages (vt, vb), its neighbours
 // (tl, tr along the top row, bu, bd along the bottom column; 0 outside the array) and g.
 template <bool YAK>
@@ -154,8 +154,13 @@ __device__ __forceinline__ void cell_residual_vals(const Grid& gr, int i, int j,
     dgf = 0.f;
   }
   if (YAK) negative_bias(gr, dv, cur, dg, dgf);
-  ft = fma(-gr.gt, tl + tr, fma(dt, vt, cur));
-  if (j == 0) ft = fma(-gr.g_src, vin_i, ft);
+  // the first column has no left neighbour but the source term: the same two instructions
+  // on other operands (x + y as 1 x + y), because a third one, predicated off elsewhere,
+  // would still take its turn on the FP64 pipe
+  const bool f = (j == 0);
+  const double base = fma(dt, vt, cur);
+  const double s = fma(f ? -gr.gt : 1.0, f ? tr : tl, f ? base : tr);
+  ft = fma(f ? -gr.g_src : -gr.gt, f ? vin_i : s, f ? s : base);
   fb = fma(-gr.gb, bu + bd, fma(db, vb, -cur));
 }
 
@@ -459,6 +464,19 @@ __device__ __forceinline__ void reduce_rows(const double* __restrict__ part, int
       h[(size_t)b * kHStride + 32 + j] = v * scale[j];
     }
   }
+}
+
+// u <- u - h_0 v_0 for a v_0 stored (and nonzero) in the first column of the top layer only
+// (the residual's sparse_f): its m entries there, by the block that has just reduced h; u
+// was written by other blocks.  The update pass then leaves v_0 out: testing every entry
+// for it took an FMA's turn on the FP64 pipe per entry (nk = 1, 1024 x 1024, 16 vectors: 148
+// us, now 118).
+__device__ __forceinline__ void subtract_sparse_v0(double* u, const double* v0,
+                                                   const double* h, int mn, int n) {
+  __syncthreads();
+  const double h0 = h[32];
+  for (int c = threadIdx.x * n; c < mn; c += blockDim.x * n)
+    u[c] = fma(-h0, v0[c], __ldcg(u + c));
 }
 
 }  // namespace
