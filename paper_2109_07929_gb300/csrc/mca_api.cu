@@ -95,7 +95,6 @@ struct mca_handle {
   int* err = nullptr;
   double *T1_64 = nullptr, *Xh_64 = nullptr, *E_64 = nullptr;
   double* fac = nullptr;          // tridiagonal factors of the paper-literal M_hat
-  int fac_ld = 0;
   __nv_bfloat16 *Xbf = nullptr, *T1bf = nullptr, *Yh = nullptr, *Eh = nullptr,
                 *El = nullptr;
   bool tc_ok = false;
@@ -341,8 +340,8 @@ int alloc_workspace(mca_handle* h) {
   MCA_TRY(dalloc(h, &h->mapbuf[0], B));
   MCA_TRY(dalloc(h, &h->mapbuf[1], B));
   h->map_of = h->mapbuf[0];
-  h->fac_ld = std::max(h->m, h->n);
-  MCA_TRY(dalloc(h, &h->fac, B * 4 * (size_t)h->fac_ld));
+  MCA_TRY(dalloc(h, &h->fac, B * mhat_fac_size(h->m, h->n)));
+  MCA_CUDA_TRY(mhat_configure());
   MCA_CUDA_TRY(cudaMemset(h->mapbuf[0], 0, B * sizeof(int)));
   MCA_CUDA_TRY(cudaMemset(h->mapbuf[1], 0, B * sizeof(int)));
   h->map_host.assign(B, 0);
@@ -605,9 +604,8 @@ int precond_apply(mca_handle* h, int precision, const double* rin, size_t rstrid
   double* zout = static_cast<double*>(zout_v);
   if (precision == MCA_PREC_MHAT) {
     cudaEvent_t t0 = prof_begin(h, s);
-    MCA_TRY(precond_mhat(h->gr, rin, rstride, zout, zstride, B, ctl, h->fac, h->fac_ld, kidx,
-                         s));
-    prof_end(h, t0, MCA_FAM_PRECOND_1, prof_k, 112.0 * (double)h->mn, 40.0 * (double)h->mn, s);
+    MCA_TRY(precond_mhat(h->gr, rin, rstride, zout, zstride, B, ctl, h->fac, kidx, s));
+    prof_end(h, t0, MCA_FAM_PRECOND_1, prof_k, 40.0 * (double)h->mn, 20.0 * (double)h->mn, s);
     return MCA_OK;
   }
   if (precision == MCA_PREC_JACOBI || precision == MCA_PREC_NONE) {

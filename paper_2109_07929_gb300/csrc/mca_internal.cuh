@@ -306,10 +306,13 @@ void launch_pack_q_bf16(const double* Q, int n, int npad, __nv_bfloat16* out_q,
                         __nv_bfloat16* out_q_lo, __nv_bfloat16* out_qt, cudaStream_t s);
 void launch_transpose64(const double* Q, int n, double* QT, cudaStream_t s);
 // paper-literal M_hat, Jacobi and identity preconditioners (k_precond_mhat.cu); fac holds
-// 4 * ld doubles per vector, ld = max(m, n)
+// mhat_fac_size(m, n) doubles per vector, built by the applies with kidx <= 0 (the first of a
+// GMRES cycle, or a single one) and used by the cycle's others
 // (the outputs carry the scale s[kidx] of the input basis vector)
+size_t mhat_fac_size(int m, int n);
+cudaError_t mhat_configure();
 int precond_mhat(const Grid& gr, const double* r, size_t rstride, double* z, size_t zstride,
-                 int B, const VecCtl* ctl, double* fac, int ld, int kidx, cudaStream_t s);
+                 int B, const VecCtl* ctl, double* fac, int kidx, cudaStream_t s);
 int precond_jacobi(const Grid& gr, const double* D, const double* r, size_t rstride, double* z,
                    size_t zstride, int B, bool none, const VecCtl* ctl, int kidx,
                    cudaStream_t s);

@@ -77,3 +77,29 @@ def test_gmres_reaches_its_tolerance(m, n, nvec, off):
         r = np.linalg.norm(rhs[v] - O.jacobian(p, cb.gmap, zero, zero) @ x[v])
         scale = np.linalg.norm(rhs[v])
         assert its[v] >= 1 and abs(r - est[v]) <= 1e-6 * r + 1e-13 * scale
+
+
+@pytest.mark.parametrize("m,n", [(2, 2), (1, 31), (32, 33), (31, 64), (65, 2), (100, 1025),
+                                 (2049, 3), (3, 2049), (1057, 40)])
+def test_mhat_line_solves_in_chunks(m, n):
+    """The paper's M_hat with every line cut into 32 chunks: lines shorter than 32 nodes, whole
+    and partly filled chunks, empty ones.  Each of the two solves is backward stable, so z_t
+    is within about 16 eps kappa of exact per solve (kappa <= (4 + a) / a: 7e-10 in all), and
+    z_b follows it; the oracle forms z_b from z_t with an error of its own of a few eps times
+    the operator's terms, 4 |z_t| / a."""
+    cb = mi.make_crossbar(m, n, 4, g_wire_bot=0.5)
+    p = cb.params
+    r = np.random.default_rng(7).standard_normal((3, 2 * m * n))
+    a = np.array([2.1e-5, 7.0e-4, 0.2])
+    prm = mca.default_params(m, n, g_wire_bot=0.5, precision=mca.PREC_MHAT, max_batch=3)
+    with mca.Solver(prm, cb.gmap) as s:
+        z = torch.empty(3, 2 * m * n, dtype=torch.float64, device=DEV)
+        s.precond_apply(a, torch.as_tensor(r, device=DEV), z)
+        z = z.cpu().numpy()
+    for v in range(3):
+        z1, z2 = O.precond_apply_block(p, None, a[v], a[v], r[v, :m * n], r[v, m * n:],
+                                       minv=lambda w: O.mhat_apply_inverse(p, a[v], a[v], w))
+        n1, n2 = np.linalg.norm(z1), np.linalg.norm(z2)
+        assert np.linalg.norm(z[v, :m * n] - z1) <= 1e-9 * n1
+        assert (np.linalg.norm(z[v, m * n:] - z2) <=
+                1e-9 * n2 + 16 * 1.1e-16 * 4 / a[v] * n1)
