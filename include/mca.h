@@ -52,7 +52,8 @@ extern "C" {
 #define MCA_ERR_UNSUPPORTED (-7)   /* precision mode not available on this device       */
 
 /* ---- precision of the preconditioner apply (Section 3.2) -------------------------- */
-#define MCA_PREC_FP64 0        /* all four eigenbasis transforms in FP64 (CUDA cores)     */
+#define MCA_PREC_FP64 0        /* all four eigenbasis transforms with FP64 results (BF16
+                                  slices on the tensor cores, summed exactly)            */
 #define MCA_PREC_BF16 1        /* all four transforms on tcgen05 tensor cores, BF16 in,
                                   FP32 accumulate                                        */
 #define MCA_PREC_BF16_SPLIT 2  /* forward transforms BF16; back transforms with the

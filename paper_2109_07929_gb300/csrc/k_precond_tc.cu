@@ -863,6 +863,20 @@ bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols,
   return r == CUDA_SUCCESS;
 }
 
+bool make_map_slices(CUtensorMap* map, const void* base, uint64_t K, uint64_t rows,
+                     uint32_t slices, uint32_t box_rows) {
+  if (!encode_available() || K % 32 != 0 || box_rows < 1 || box_rows > 256) return false;
+  cuuint64_t gdim[3] = {K, rows, slices};
+  cuuint64_t gstride[2] = {K * 2, K * 2 * rows};
+  cuuint32_t box[3] = {32, box_rows, slices};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode.load()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base),
+                               gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 // 4-D BF16 map over an NHWC activation tensor with 32 channels ([n][y][x][c], 64 bytes per
 // pixel) and a box of box_px pixels of one row of one image, 64-byte swizzle (one pixel
 // = one swizzle row).  Out-of-range boxes read zeros (the convolutions' padding).

@@ -94,6 +94,9 @@ struct mca_handle {
   int32_t* hflags_dev = nullptr;
   int* err = nullptr;
   double *T1_64 = nullptr, *Xh_64 = nullptr, *E_64 = nullptr;
+  // FP64 transforms on the tensor cores: slices of the data (rows of m x n and of n x m
+  // matrices share a buffer) and of the eigenvector matrices
+  SlicedOperand opA_mn, opA_nm, opQrT, opQcT, opQr, opQc;
   double* fac = nullptr;          // tridiagonal factors of the paper-literal M_hat
   __nv_bfloat16 *Xbf = nullptr, *T1bf = nullptr, *Yh = nullptr, *Eh = nullptr,
                 *El = nullptr;
@@ -308,6 +311,33 @@ int setup_tc(mca_handle* h) {
   return MCA_OK;
 }
 
+// Slices of the eigenvector matrices and room for the data's, for the FP64 transforms.
+int setup_sliced(mca_handle* h) {
+  if (!tc::encode_available()) {
+    set_error("cuTensorMapEncodeTiled unavailable");
+    return MCA_ERR_UNSUPPORTED;
+  }
+  const int m = h->m, n = h->n;
+  const int am = 2 * h->Bmax * m, an = 2 * h->Bmax * n;   // rows of the data operands
+  __nv_bfloat16* buf = nullptr;
+  int* exps = nullptr;
+  MCA_TRY(dalloc(h, &buf, std::max(sliced_elems(am, n), sliced_elems(an, m))));
+  MCA_TRY(dalloc(h, &exps, (size_t)std::max(am, an)));
+  MCA_TRY(make_sliced(&h->opA_mn, buf, exps, am, n, true));
+  MCA_TRY(make_sliced(&h->opA_nm, buf, exps, an, m, true));
+  const struct { SlicedOperand* op; const double* q; int k; } qs[] = {
+      {&h->opQrT, h->QrT, n}, {&h->opQcT, h->QcT, m}, {&h->opQr, h->Qr, n}, {&h->opQc, h->Qc, m}};
+  for (const auto& q : qs) {
+    MCA_TRY(dalloc(h, &buf, sliced_elems(q.k, q.k)));
+    MCA_TRY(dalloc(h, &exps, (size_t)q.k));
+    MCA_TRY(make_sliced(q.op, buf, exps, q.k, q.k, false));
+    launch_slice_rows(q.q, BlkAddr{0, 0, (size_t)q.k}, q.k, *q.op, q.k, nullptr, 0);
+    count_launches(1);
+  }
+  MCA_CUDA_TRY(cudaGetLastError());
+  return MCA_OK;
+}
+
 int alloc_workspace(mca_handle* h) {
   const size_t B = h->Bmax, n2 = h->n2, mn = h->mn;
   const size_t kv = h->restart + 1;
@@ -352,6 +382,7 @@ int alloc_workspace(mca_handle* h) {
     MCA_TRY(dalloc(h, &h->T1_64, B * n2));
     MCA_TRY(dalloc(h, &h->Xh_64, B * n2));
     MCA_TRY(dalloc(h, &h->E_64, B * n2));
+    MCA_TRY(setup_sliced(h));
   }
   MCA_CUDA_TRY(cudaHostAlloc(&h->hflags, 64 * sizeof(int32_t), cudaHostAllocMapped));
   MCA_CUDA_TRY(cudaHostGetDevicePointer(&h->hflags_dev, h->hflags, 0));
@@ -621,27 +652,29 @@ int precond_apply(mca_handle* h, int precision, const double* rin, size_t rstrid
   if (precision == MCA_PREC_FP64) {
     if (!h->T1_64) return MCA_ERR_UNSUPPORTED;
     const double f_r = 4.0 * m * (double)n * n, f_c = 4.0 * n * (double)m * m;
+    // O[blk][c][r] = sum_k A[blk][r][k] Q[c][k] for the blocks of B vectors
+    auto transform = [&](const double* A, BlkAddr a, const SlicedOperand& op,
+                         const SlicedOperand& q, double* O, BlkAddr o, int R, int K) {
+      launch_slice_rows(A, a, R, op, 2 * B * R, ctl, s);
+      count_launches(1 + launch_gemm_sliced(op, q, O, o, B, R, K, ctl, h->err, s));
+    };
     BlkAddr a1{rstride, mn, (size_t)n}, o1{2 * mn, mn, (size_t)m};
     cudaEvent_t t0 = prof_begin(h, s);
-    launch_gemm64_tstore(rin, a1, h->QrT, h->T1_64, o1, B, m, n, n, ctl, s);
-    count_launches(1);
+    transform(rin, a1, h->opA_mn, h->opQrT, h->T1_64, o1, m, n);
     prof_end(h, t0, MCA_FAM_PRECOND_1, prof_k, 32.0 * mn, f_r, s);
     BlkAddr a2{2 * mn, mn, (size_t)m}, o2{2 * mn, mn, (size_t)n};
     t0 = prof_begin(h, s);
-    launch_gemm64_tstore(h->T1_64, a2, h->QcT, h->Xh_64, o2, B, n, m, m, ctl, s);
-    count_launches(1);
+    transform(h->T1_64, a2, h->opA_nm, h->opQcT, h->Xh_64, o2, n, m);
     launch_modes_2x2_f64(h->Xh_64, h->mu, h->nu, m, n, ctl, B, kidx, s);
     count_launches(1);
     prof_end(h, t0, MCA_FAM_PRECOND_2, prof_k, 64.0 * mn, f_c, s);
     BlkAddr a3{2 * mn, mn, (size_t)n}, o3{2 * mn, mn, (size_t)m};
     t0 = prof_begin(h, s);
-    launch_gemm64_tstore(h->Xh_64, a3, h->Qr, h->E_64, o3, B, m, n, n, ctl, s);
-    count_launches(1);
+    transform(h->Xh_64, a3, h->opA_mn, h->opQr, h->E_64, o3, m, n);
     prof_end(h, t0, MCA_FAM_PRECOND_3, prof_k, 32.0 * mn, f_r, s);
     BlkAddr a4{2 * mn, mn, (size_t)m}, o4{zstride, mn, (size_t)n};
     t0 = prof_begin(h, s);
-    launch_gemm64_tstore(h->E_64, a4, h->Qc, zout, o4, B, n, m, m, ctl, s);
-    count_launches(1);
+    transform(h->E_64, a4, h->opA_nm, h->opQc, zout, o4, n, m);
     prof_end(h, t0, MCA_FAM_PRECOND_4, prof_k, 32.0 * mn, f_c, s);
     MCA_CUDA_TRY(cudaGetLastError());
     return MCA_OK;

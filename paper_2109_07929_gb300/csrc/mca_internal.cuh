@@ -318,18 +318,13 @@ int precond_jacobi(const Grid& gr, const double* D, const double* r, size_t rstr
                    cudaStream_t s);
 // element-wise out = a - b on nvec vectors of n2 doubles (k_krylov.cu)
 void launch_sub(const double* a, const double* b, double* out, size_t n2, int B, cudaStream_t s);
-// FP64 preconditioner (k_precond64.cu)
-// Block-transposed GEMM used by all four eigenbasis transforms:
-//   O[blk][c][r] = sum_k A[blk][r][k] * Bm[c][k]   (r < R, c < C, k < K)
-// with blk = 2*b + layer; A block blk starts at A + b*a.bs + layer*a.ls (row stride K),
-// O block blk starts at O + b*o.bs + layer*o.ls (row stride o.ld along c).
+// FP64 preconditioner (k_precond64.cu; its GEMM is declared in precond_tc.h): addressing of
+// the blocks blk = 2 b + layer of an operand or output, at base + b bs + layer ls.
 struct BlkAddr {
   size_t bs;   // elements between batch entries
   size_t ls;   // elements between the two layers of one entry
-  size_t ld;   // leading dimension (A: row stride; O: stride between c)
+  size_t ld;   // leading dimension (operand: row stride; output: stride between columns)
 };
-void launch_gemm64_tstore(const double* A, BlkAddr a, const double* Bm, double* O, BlkAddr o,
-                          int B, int R, int K, int C, const VecCtl* ctl, cudaStream_t s);
 // Per-mode 2x2 inverse of eq. (P) in place on X_hat[b][layer][i'][k'] (m x n), times the
 // scale s[kidx] of the (unnormalised) input basis vector.
 void launch_modes_2x2_f64(double* Xh, const double* mu, const double* nu, int m, int n,

@@ -43,6 +43,10 @@ bool encode_available();
 // box_k: 64 (single-word GEMMs) or 32 (split GEMMs)
 bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols,
               uint32_t box_rows, uint32_t box_k);
+// 3-D map over BF16 slices [slices][rows][K] (K a multiple of 32), box = 32 of K x box_rows x
+// every slice (64-byte swizzle; rows beyond the last read zero)
+bool make_map_slices(CUtensorMap* map, const void* base, uint64_t K, uint64_t rows,
+                     uint32_t slices, uint32_t box_rows);
 // 4-D map over an NHWC BF16 tensor with 32 channels, box = box_px pixels of one row
 // (64-byte swizzle; out-of-range elements read zero)
 bool make_map_nhwc32(CUtensorMap* map, const void* base, uint64_t W, uint64_t H, uint64_t N,
@@ -69,4 +73,24 @@ void cast_pad(const double* x, size_t xstride, __nv_bfloat16* xbf, int m, int n,
               int np, int B, cudaStream_t s);
 
 }  // namespace tc
+
+// ---- FP64 GEMM on the tensor cores (k_precond64.cu) ----------------------------------------
+// An operand cut into BF16 slices: `rows` rows of K entries, row exponents and the TMA map.
+struct SlicedOperand {
+  CUtensorMap map;
+  __nv_bfloat16* buf = nullptr;
+  int* exps = nullptr;
+  int rows = 0, K = 0, Kp = 0;
+};
+// BF16 elements the slices of rows x K entries take
+size_t sliced_elems(size_t rows, int K);
+// Describe an operand (A: data, else the matrix Bm) whose slices live in buf.
+int make_sliced(SlicedOperand* op, __nv_bfloat16* buf, int* exps, int rows, int K, bool is_a);
+// Slices and exponents of the first `rows` rows: row r of block blk = 2 b + layer (R rows per
+// block) starts at A + b a.bs + layer a.ls + r a.ld; blocks of inactive vectors are skipped.
+void launch_slice_rows(const double* A, BlkAddr a, int R, const SlicedOperand& op, int rows,
+                       const VecCtl* ctl, cudaStream_t s);
+// O[blk][c][r] = sum_k A[blk][r][k] Bm[c][k] for 2 B blocks; returns the launches made.
+int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, double* O, BlkAddr o,
+                       int B, int R, int C, const VecCtl* ctl, int* err, cudaStream_t s);
 }  // namespace mca

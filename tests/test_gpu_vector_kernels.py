@@ -103,3 +103,31 @@ def test_mhat_line_solves_in_chunks(m, n):
         assert np.linalg.norm(z[v, :m * n] - z1) <= 1e-9 * n1
         assert (np.linalg.norm(z[v, m * n:] - z2) <=
                 1e-9 * n2 + 16 * 1.1e-16 * 4 / a[v] * n1)
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 33), (5, 130), (129, 65), (64, 257), (2, 4100)])
+def test_fp64_preconditioner_in_slices(m, n):
+    """The FP64 transforms on BF16 slices: ragged tiles and K, and (4100) a K beyond one FP32
+    accumulator.  P z = r within the eigenvectors' own accuracy (1e-9, the bar of their parity
+    test) of |P| |z|; scaling r by 2^-980 scales z exactly (every row's slices are relative to
+    its exponent); a NaN reaches the output."""
+    cb = mi.make_crossbar(m, n, 4)
+    p = cb.params
+    rng = np.random.default_rng(7)
+    r = rng.uniform(0.5, 1.0, (2, 2 * m * n)) * rng.choice([-1.0, 1.0], (2, 2 * m * n))
+    r[1, : m * n] *= 10.0 ** rng.uniform(-8, 0, m * n)
+    a = np.array([2.1e-5, 0.2])
+    with mca.Solver(mca.default_params(m, n, precision=mca.PREC_FP64, max_batch=2), cb.gmap) as s:
+        rd = torch.as_tensor(r, device=DEV)
+        z, zs, zn = (torch.empty_like(rd) for _ in range(3))
+        s.precond_apply(a, rd, z)
+        s.precond_apply(a, rd * 2.0 ** -980, zs)
+        rd[0, 0] = float("nan")
+        s.precond_apply(a, rd, zn)
+    assert torch.equal(zs, z * 2.0 ** -980)
+    assert bool(torch.isnan(zn[0]).any()) and torch.equal(zn[1], z[1])
+    z = z.cpu().numpy()
+    for v in range(2):
+        P = O.precond_matrix(p, a[v], a[v])
+        size = 5.0 + 2 * a[v]                      # |P| <= 4 g + 2 a, plus the terminations
+        assert np.linalg.norm(P @ z[v] - r[v]) <= 1e-9 * size * np.linalg.norm(z[v])
