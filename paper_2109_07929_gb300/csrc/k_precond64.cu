@@ -54,13 +54,13 @@ constexpr int kOzKMax = 4096;     // largest K summed in one FP32 accumulator
 constexpr int kBadRow = 0x7FFFFFFF;   // exponent of a row with an infinity or a NaN
 constexpr int kZeroRow = -0x7FFFFFFF; // and of a row of zeros
 
-// Row slicing: a warp per row.  out[s][row][k] (BF16, K padded to Kp with zeros, `rows` rows
-// in all) and exps[row].  Row r of block blk = 2 b + layer starts at A + b a.bs + layer a.ls
-// + r a.ld.  Integer arithmetic only: the entry's mantissa shifted to a 56-bit fixed-point
+// Row slicing: a warp per row, `rows` of them (of the batch at hand; the operand holds
+// plane / Kp).  out[s][row][k] (BF16, K padded to Kp with zeros) and exps[row].  Row r of
+// block blk = 2 b + layer starts at A + b a.bs + layer a.ls + r a.ld.  Integer arithmetic only: the entry's mantissa shifted to a 56-bit fixed-point
 // number in units of 2^(e - 54), its digits taken from the low end with a carry.
 __global__ void __launch_bounds__(256)
 k_slice_rows(const double* __restrict__ A, BlkAddr a, int R, int K, int Kp, int rows,
-             const VecCtl* __restrict__ ctl, __nv_bfloat16* __restrict__ out,
+             size_t plane, const VecCtl* __restrict__ ctl, __nv_bfloat16* __restrict__ out,
              int* __restrict__ exps) {
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -88,7 +88,6 @@ k_slice_rows(const double* __restrict__ A, BlkAddr a, int R, int K, int Kp, int 
   }
   const int E = (int)(top >> 20);                    // biased exponent of the largest entry
   if (lane == 0) exps[row] = bad ? kBadRow : (any ? E - 1023 - (low ? 512 : 0) : kZeroRow);
-  const size_t plane = (size_t)rows * Kp;
   __nv_bfloat16* o = out + (size_t)row * Kp;
   for (int k0 = 2 * lane; k0 < Kp; k0 += 64) {
     uint32_t w[kSlices] = {};
@@ -332,7 +331,8 @@ int make_sliced(SlicedOperand* op, __nv_bfloat16* buf, int* exps, int rows, int 
 
 void launch_slice_rows(const double* A, BlkAddr a, int R, const SlicedOperand& op, int rows,
                        const VecCtl* ctl, cudaStream_t s) {
-  k_slice_rows<<<(rows + 7) / 8, 256, 0, s>>>(A, a, R, op.K, op.Kp, rows, ctl, op.buf, op.exps);
+  k_slice_rows<<<(rows + 7) / 8, 256, 0, s>>>(A, a, R, op.K, op.Kp, rows,
+                                              (size_t)op.rows * op.Kp, ctl, op.buf, op.exps);
 }
 
 int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, double* O, BlkAddr o,

@@ -131,3 +131,18 @@ def test_fp64_preconditioner_in_slices(m, n):
         P = O.precond_matrix(p, a[v], a[v])
         size = 5.0 + 2 * a[v]                      # |P| <= 4 g + 2 a, plus the terminations
         assert np.linalg.norm(P @ z[v] - r[v]) <= 1e-9 * size * np.linalg.norm(z[v])
+
+
+@pytest.mark.parametrize("m,n,nvec", [(5, 130, 1), (129, 65, 2)])
+def test_fp64_preconditioner_of_part_of_a_batch(m, n, nvec):
+    """Fewer vectors than the handle holds: the same values as in a handle made for them."""
+    cb = mi.make_crossbar(m, n, 4)
+    r = np.random.default_rng(8).uniform(-1.0, 1.0, (nvec, 2 * m * n))
+    zs = []
+    for mb in (nvec, 3):
+        pr = mca.default_params(m, n, precision=mca.PREC_FP64, max_batch=mb)
+        with mca.Solver(pr, cb.gmap) as s:
+            rd = torch.as_tensor(r, device=DEV)
+            zs.append(torch.empty_like(rd))
+            s.precond_apply(np.full(nvec, 2.1e-5), rd, zs[-1])
+    assert torch.equal(zs[0], zs[1])
