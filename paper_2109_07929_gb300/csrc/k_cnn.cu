@@ -10,28 +10,35 @@
 // a K x K convolution with dilation d and zero padding d (K - 1) / 2 (output size = input
 // size), plus bias and an optional leaky ReLU (slope 0.1).
 //
-// Convolutions are implicit GEMMs on the tcgen05 tensor cores:
-//   forward  out[p][co] = sum_t sum_ci W[t][co][ci] x[p + off_t][ci]: a CTA owns 128
-//            pixels of one image row (M = 128, TMEM lane = pixel) and all output channels
-//            (N = 16 or 32); per kernel row ky one pipeline stage holds the shifted input
-//            row segment (128 + (K - 1) d pixels, out-of-range pixels read as zero: the
-//            padding) in the K-major layout without swizzle, whose 16-byte pixel rows let
-//            the K taps of that row start at any pixel offset of the same segment, plus the
-//            row's K weight tiles; two MMAs (K = 16 channels each) per tap accumulate;
+// Convolutions are implicit GEMMs on the tcgen05 tensor cores, each in two forms:
+//   forward  out[p][co] = sum_t sum_ci W[t][co][ci] x[p + off_t][ci].  k_conv_taps (32 output
+//            channels, K >= 5): four taps' weights are the rows (M = 4 x 32), the pixels of an
+//            input row the columns, and the drain adds the four taps' shifted rows.
+//            k_conv_tc (16 output channels, small kernels, dilations beyond k_conv_taps'
+//            shared memory): a CTA owns 128 pixels of one image row (M = 128, TMEM lane =
+//            pixel) and all output channels (N = 16 or 32); per kernel row ky one pipeline
+//            stage holds the shifted input row segment (128 + (K - 1) d pixels, out-of-range
+//            pixels read as zero: the padding) in the K-major layout without swizzle, whose
+//            16-byte pixel rows let the K taps of that row start at any pixel offset of the
+//            same segment, plus the row's K weight tiles; two MMAs (K = 16 channels each) per
+//            tap accumulate;
 //   backward data is the same operation on the output gradient with the taps flipped and
 //            the channel roles swapped (mca_cnn_prep_weights builds both weight tiles), with
 //            the activation derivative of the layer below applied in the epilogue;
-//   weight gradient gW[t][co][ci] = sum_p gz[p][co] x[p + off_t][ci]: M = 4 taps x 32 input
-//            channels, N = 32 output channels, K = pixels; both operands come straight from
-//            the NHWC tensors as MN-major tiles (64 consecutive pixels of a row per stage),
-//            a CTA covers one group of 4 taps over a block of rows and writes FP32 partial
-//            sums that a second kernel adds in a fixed order.
+//   weight gradient gW[t][co][ci] = sum_p gz[p][co] x[p + off_t][ci], K = pixels, both
+//            operands straight from the NHWC tensors as MN-major tiles.  k_wgrad_rows (K from 5
+//            to 13): rows of the gradient against rows of the input, all taps of a kernel row
+//            at once.  k_conv_wgrad_tc (the other kernel sizes): M = 4 taps x 32 input
+//            channels, N = 32 output channels, 64 consecutive pixels of a row per stage, a CTA
+//            covers one group of 4 taps over a block of rows.  Both write FP32 partial sums
+//            that a second kernel adds in a fixed order.
 // Every mbarrier wait is bounded; an expired wait sets the module's error flag (read and
 // cleared by mca_cnn_check) and the CTA leaves after freeing its TMEM.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -265,6 +272,348 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
   }
 }
 
+// ---- convolution with 32 output channels, weights as the M operand ----------------------
+//
+// k_conv_tc multiplies 128 pixels by 32 output channels per MMA: it reads 4 KB of pixels from
+// shared memory for 16 clocks of work, and fills and drains its pipeline for every 128 pixels
+// with the tensor core idle (347 TFLOP/s).  Here M holds 4 neighbouring taps of a kernel row x
+// 32 output channels and N the pixels:
+//   D_q[co][u] = sum_ky sum_g sum_ci W[ky][4 g + q][co][ci] x[y + (ky - r) d][b + u + 4 g d][ci]
+// for q = 0 .. 3, b = x0 - r d: the taps of group g see a window shifted by 4 g d pixels (16-byte
+// pixel rows without swizzle: any start), so that all groups add to one accumulator, and
+//   out[co][x0 + p] = sum_q D_q[co][p + q d]
+// is left to the epilogue: N = P + 3 d columns for P pixels.  Taps beyond the kernel row read
+// as zero weights (TMA bounds; where K is no multiple of 4, an infinity or NaN in x therefore
+// reaches up to 3 output pixels more per row than its window); input rows outside the image
+// are left out.
+// One persistent CTA per SM walks the tiles (P pixels of one image row): per stage, warp 0
+// brings in a kernel row's weights (TMA) and 8 warps its input row, warp 1 issues 2 G MMAs of
+// 128 x N x 16 into one of two accumulators, and 8 warps drain the other one, 64 pixels at a
+// time.  The input rows go through 16-byte asynchronous copies: a TMA box of one 8-channel
+// plane consists of 16-byte rows, and 700 of those per stage took three times its MMAs.
+// Bound: the input rows' copies and the drain, each about 1200 clocks per stage against 430
+// of MMAs.  32 images of 256 x 256, 11 x 11, dilation 4: 1495 us, now 760 (one CTA per tile
+// with the drain exposed: 1081; persistent with TMA input rows: 828).
+constexpr int kTapM = 4;               // taps per M tile
+constexpr int kTapPad = 36;            // floats per pixel of the epilogue's staging rows
+constexpr int kTapChunk = 64;          // pixels drained at a time
+constexpr int kTapMaxStages = 8;
+constexpr int kTapDrain = 256;         // threads of the drain (warps 2 .. 9)
+constexpr int kTapCopy = 256;          // threads of the input rows (warps 10 .. 17)
+constexpr int kTapThreads = 64 + kTapDrain + kTapCopy;
+constexpr int kTapStaging = kTapM * kTapChunk * kTapPad * 4;
+
+struct TapPlan {
+  int G, P, N;                         // tap groups, pixels per tile, accumulator columns
+  int seg, lbo;                        // input row: pixels, bytes per plane of 8 channels
+  int wb, rb, stage, stages;           // bytes of a stage's weights and input row
+  int smem;
+};
+
+// False where the old form is the better one (or the only one that fits).
+bool tap_plan(int K, int d, int W, TapPlan& p) {
+  if (K < 5) return false;             // a row of 1 or 3 taps would leave M mostly zero
+  p.G = (K + kTapM - 1) / kTapM;
+  long best = -1;
+  for (int P = 16; P <= 240; P += 16) {
+    const int N = (P + (kTapM - 1) * d + 15) / 16 * 16;
+    if (N > 256) break;
+    const long cost = (long)((W + P - 1) / P) * (N + 16);
+    if (best < 0 || cost < best) {
+      best = cost;
+      p.P = P;
+      p.N = N;
+    }
+  }
+  if (best < 0) return false;
+  p.seg = p.N + kTapM * (p.G - 1) * d;
+  // planes 2 x 16 bytes apart modulo 128: the copies of two pixels' four planes hit
+  // different banks
+  p.lbo = ((p.seg + 5) / 8 * 8 + 2) * 16;
+  p.rb = (4 * p.lbo + 1023) / 1024 * 1024;
+  p.wb = p.G * kTapM * kC * kC * 2;
+  p.stage = p.wb + p.rb;
+  const int room = 224 * 1024 - kTapStaging;
+  p.stages = room / p.stage < kTapMaxStages ? room / p.stage : kTapMaxStages;
+  if (p.stages < 2) return false;
+  p.smem = p.stages * p.stage + kTapStaging + 512 + 1024;
+  return true;
+}
+
+struct TapArgs {
+  int H, W, K, d, r;
+  int xt, tiles;                       // tiles per image row and in all
+  int cout;
+  const __nv_bfloat16* x;
+  const float* bias;
+  int act, backward;
+  const __nv_bfloat16* yprev;
+  __nv_bfloat16* out;
+  float* out32;
+  TapPlan plan;
+};
+
+// 16 bytes to shared memory, zeros when !ok (src must be readable memory either way)
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
+}
+
+// At most LEFT of this thread's newest copy groups may still be in flight.
+template <int LEFT>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+__global__ void __launch_bounds__(kTapThreads, 1)
+k_conv_taps(const __grid_constant__ CUtensorMap tmW, TapArgs a) {
+  const TapPlan& P = a.plan;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int S = P.stages;
+  float* stg = reinterpret_cast<float*>(smem + S * P.stage);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * P.stage + kTapStaging);
+  uint64_t* empty = full + kTapMaxStages;
+  uint64_t* tfull = empty + kTapMaxStages;           // [2] accumulator complete
+  uint64_t* tempty = tfull + 2;                      // [2] accumulator drained
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  volatile uint32_t& dead = tmem_slot[1];            // a drain warp's wait gave up
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int d = a.d;
+  // tile t: P pixels from x0 of row y of image n, and the kernel rows that meet the image
+  auto decode = [&](int t, int& n, int& y, int& x0, int& k0, int& k1) {
+    const int row = t / a.xt;
+    x0 = (t - row * a.xt) * P.P;
+    n = row / a.H;
+    y = row - n * a.H;
+    k0 = max(0, a.r - y / d);
+    k1 = min(a.K - 1, a.r + (a.H - 1 - y) / d);
+  };
+  if (threadIdx.x == 0) {
+    dead = 0;
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 1 + kTapCopy);
+      mbar_init(&empty[s], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&tfull[q], 1);
+      mbar_init(&tempty[q], kTapDrain / 32);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)), "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+        int n, y, x0, k0, k1;
+        decode(t, n, y, x0, k0, k1);
+        for (int ky = k0; ky <= k1; ++ky, ++it) {
+          const int s = it % S;
+          if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u)) {
+            atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+            ok = false;
+            break;
+          }
+          uint8_t* st = smem + s * P.stage;
+          mbar_expect_tx(&full[s], (uint32_t)P.wb);
+          for (int g = 0; g < P.G; ++g)
+            tma_load_4d(st + g * kTapM * kC * kC * 2, &tmW, 0, 0, g * kTapM, ky, &full[s]);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16(kTapM * kC, P.N);
+      int it = 0, tl = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tl) {
+        int n, y, x0, k0, k1;
+        decode(t, n, y, x0, k0, k1);
+        const int acc = tl & 1;
+        if (!mbar_wait(&tempty[acc], ((uint32_t)(tl >> 1) & 1u) ^ 1u)) {
+          atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t dst = tmem + (uint32_t)(acc * 256);
+        for (int ky = k0; ky <= k1; ++ky, ++it) {
+          const int s = it % S;
+          if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u)) {
+            atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint8_t* wt = smem + s * P.stage;
+          const uint8_t* row = wt + P.wb;
+          for (int g = 0; g < P.G; ++g) {
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+              umma(dst, sw64_desc(wt + g * kTapM * kC * kC * 2 + kk * 32),
+                   kmajor_noswz_desc(row + kTapM * g * d * 16 + kk * 2 * P.lbo, P.lbo, 128), idesc,
+                   (ky > k0 || g > 0 || kk > 0) ? 1u : 0u);
+          }
+          umma_commit(&empty[s]);
+        }
+        if (ok) umma_commit(&tfull[acc]);
+      }
+    }
+  } else if (warp >= 2 + kTapDrain / 32) {
+    // ---------------- input rows: pixel-major 16-byte copies into the four planes; a row is
+    // reported one row later, when its copies have landed (the slot of row `it` is free once
+    // row it - S is consumed, and S >= 2; reporting three rows later left the MMAs too few
+    // rows ahead: 257 against 202 us per layer at 8 images of 256 x 256)
+    const int tid = threadIdx.x - 64 - kTapDrain;
+    constexpr int lag = 1;
+    auto report = [&](int it) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[it % S]))
+                   : "memory");
+    };
+    int it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+      int n, y, x0, k0, k1;
+      decode(t, n, y, x0, k0, k1);
+      for (int ky = k0; ky <= k1; ++ky, ++it) {
+        const int s = it % S;
+        if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u)) {
+          atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+          ok = false;
+          break;
+        }
+        const uint32_t dst = smem_u32(smem + s * P.stage + P.wb);
+        const __nv_bfloat16* src =
+            a.x + ((size_t)n * a.H + (y + (ky - a.r) * d)) * a.W * kC;
+        for (int e = tid; e < P.seg * 4; e += kTapCopy) {
+          const int px = e >> 2, kc = e & 3, xx = x0 - a.r * d + px;
+          const bool in = xx >= 0 && xx < a.W;
+          copy16_async(dst + kc * P.lbo + px * 16, src + (size_t)(in ? xx : 0) * kC + kc * 8, in);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (it >= lag) {
+          copies_wait<lag>();
+          report(it - lag);
+        }
+      }
+    }
+    copies_wait<0>();                          // (also after a timeout: no copy outlives the CTA)
+    if (ok)
+      for (int r = it - lag > 0 ? it - lag : 0; r < it; ++r) report(r);
+  } else {
+    // ---------------- drain: 64 pixels at a time, the four taps' accumulators to shared memory
+    // as [q][pixel][channel], shifted by q d (a warp reads the lanes of tap warp % 4), then one
+    // thread per pixel and 8 channels adds them
+    const int q = warp & 3, hf = (warp - 2) >> 2, tid = threadIdx.x - 64;
+    const int pl = tid >> 2, c8 = (tid & 3) * 8;
+    float bias[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      bias[c] = (!a.backward && a.bias && c8 + c < a.cout) ? a.bias[c8 + c] : 0.f;
+    const bool gate = a.backward && a.act && a.yprev;
+    int tl = 0;
+    for (int t = blockIdx.x; t < a.tiles; t += gridDim.x, ++tl) {
+      int n, y, x0, k0, k1;
+      decode(t, n, y, x0, k0, k1);
+      const int acc = tl & 1;
+      const bool have = __all_sync(0xffffffffu,
+                                   mbar_wait(&tfull[acc], (uint32_t)(tl >> 1) & 1u) ? 1 : 0) != 0;
+      if (!have && lane == 0) {
+        atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+        dead = 1;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kTapDrain) : "memory");
+      if (dead) break;                 // (all 8 warps: a wait that gave up)
+      tc_fence_after();
+      for (int p0 = 0; p0 < P.P; p0 += kTapChunk) {
+        const int p = p0 + pl, x = x0 + p;
+        const bool in = p < P.P && x < a.W;
+        const size_t px = ((size_t)n * a.H + y) * a.W + x;
+        uint4 yp = {};
+        if (gate && in) yp = *reinterpret_cast<const uint4*>(a.yprev + px * kC + c8);
+        // columns p0 + q d .. + 63 of this tap, in 16-column blocks
+        const int first = p0 + q * d;
+        const int c1 = min(P.N, first + kTapChunk);
+        for (int c0 = first / 16 * 16 + hf * 16; c0 < c1; c0 += 32) {
+          uint32_t v[16];
+          tmem_ld16(tmem + (uint32_t)(acc * 256 + c0) + ((uint32_t)(q * 32) << 16), v);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int u = c0 + j - first;
+            if (u >= 0 && u < kTapChunk)
+              stg[(q * kTapChunk + u) * kTapPad + lane] = __uint_as_float(v[j]);
+          }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kTapDrain) : "memory");
+        if (in) {
+          float o[8] = {};
+#pragma unroll
+          for (int k = 0; k < kTapM; ++k) {
+            const float4* src =
+                reinterpret_cast<const float4*>(stg + (k * kTapChunk + pl) * kTapPad + c8);
+            const float4 u = src[0], w = src[1];
+            o[0] += u.x; o[1] += u.y; o[2] += u.z; o[3] += u.w;
+            o[4] += w.x; o[5] += w.y; o[6] += w.z; o[7] += w.w;
+          }
+          const __nv_bfloat16* ypb = reinterpret_cast<const __nv_bfloat16*>(&yp);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            if (gate) {
+              o[c] *= (__bfloat162float(ypb[c]) > 0.f) ? 1.f : 0.1f;
+            } else if (!a.backward) {
+              o[c] += bias[c];
+              if (a.act) o[c] = leaky(o[c]);
+            }
+            if (c8 + c >= a.cout) o[c] = 0.f;
+          }
+          if (a.out) {
+            uint4 pk;
+            uint32_t* w32 = reinterpret_cast<uint32_t*>(&pk);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const __nv_bfloat162 b2 = __floats2bfloat162_rn(o[2 * c], o[2 * c + 1]);
+              w32[c] = *reinterpret_cast<const uint32_t*>(&b2);
+            }
+            *reinterpret_cast<uint4*>(a.out + px * kC + c8) = pk;
+          }
+          if (a.out32) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              if (c8 + c < a.cout) a.out32[px * a.cout + c8 + c] = o[c];
+          }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kTapDrain) : "memory");
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[acc]))
+                     : "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+  }
+}
+
 // ---- weight gradient ------------------------------------------------------------------
 
 struct WgLayout {
@@ -398,6 +747,144 @@ k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   }
 }
 
+// ---- weight gradient, rows against rows --------------------------------------------------
+//
+// k_conv_wgrad_tc brings 20 KB through shared memory per 64 pixels for 4 MMAs of 16 clocks'
+// work: it is bound by L2 reads (201 TFLOP/s).  Here a CTA owns one kernel column kx and
+// multiplies 4 gradient rows y + j d (M = 4 x 32 output channels) by the K + 3 input rows
+// y + (i - r) d shifted by (kx - r) d pixels (N = 32 (K + 3) input channels, at most the 512
+// TMEM columns):
+//   D[(j, co)][(i, ci)] = sum_x gz[y + j d][x][co] x[y + (i - r) d][x + (kx - r) d][ci],
+// whose blocks i = j + ky are the four rows' parts of tap (ky, kx): 4 K of 4 (K + 3) blocks
+// are used, and 72 KB per 64 pixels feed 900 clocks of MMAs (K = 11).  D accumulates over a
+// share of the images' row blocks; the epilogue adds the four diagonals and writes one
+// partial sum per CTA.  Rows beyond the image read zero (a NaN in x reaches, where the row
+// blocks do not divide H, taps whose own gradient rows all lie outside).
+// Bound: L2 reads and MMA issue.  32 images of 256 x 256, 11 x 11, dilation 4: 2583 us, now
+// 660.
+constexpr int kWrJ = 4;                                 // gradient rows per CTA step
+constexpr int kWrRow = kWgPix * kC * 2;                 // 64 pixels of a row: 4 KB
+constexpr int kWrMaxK = 512 / kC - (kWrJ - 1);          // 13
+constexpr int kWrStages = 3;                            // (2 where 3 do not fit: K = 13)
+// Row-block chunks per partial sum: 256 MMA steps per accumulator, as many as the other form
+// takes on 256-pixel rows (the tensor core's FP32 sums lose about a rounding per step)
+constexpr int kWrItems = 64;
+
+struct WrArgs {
+  int H, K, d, r;
+  int stages;
+  int blocks;            // row blocks of one image
+  int items;             // N * blocks * nxc
+  int nxc;               // 64-pixel chunks per row
+  float* part;           // [chunk][t][ci 32][co 32]
+};
+
+__global__ void __launch_bounds__(128, 1)
+k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
+             WrArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int rows = a.K + kWrJ - 1, stage = (rows + kWrJ) * kWrRow, S = a.stages;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage);
+  uint64_t* empty = full + S;
+  uint64_t* accum = empty + S;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kx = blockIdx.x, chunk = blockIdx.y;
+  const int it0 = (int)((long long)a.items * chunk / gridDim.y);
+  const int steps = (int)((long long)a.items * (chunk + 1) / gridDim.y) - it0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accum, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)), "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  if (threadIdx.x == 0) {
+    for (int it = 0; it < steps; ++it) {
+      const int s = it % S;
+      if (!mbar_wait(&empty[s], ((uint32_t)(it / S) & 1u) ^ 1u)) {
+        atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+        break;
+      }
+      uint8_t* st = smem + s * stage;
+      mbar_expect_tx(&full[s], (uint32_t)stage);
+      const int item = it0 + it;
+      const int xc = item % a.nxc, rb = item / a.nxc;
+      const int n = rb / a.blocks, blk = rb - n * a.blocks;
+      const int y = blk / a.d * kWrJ * a.d + blk % a.d, x0 = xc * kWgPix;
+      for (int j = 0; j < kWrJ; ++j)
+        tma_load_4d(st + j * kWrRow, &tmG, 0, x0, y + j * a.d, n, &full[s]);
+      for (int i = 0; i < rows; ++i)
+        tma_load_4d(st + (kWrJ + i) * kWrRow, &tmX, 0, x0 + (kx - a.r) * a.d,
+                    y + (i - a.r) * a.d, n, &full[s]);
+    }
+  } else if (threadIdx.x == 32) {
+    const int n1 = rows * kC < 256 ? rows * kC : 256, n2 = rows * kC - n1;
+    const uint32_t id1 = idesc_bf16_mn(128, n1), id2 = idesc_bf16_mn(128, n2 > 0 ? n2 : 32);
+    bool ok = true;
+    for (int it = 0; it < steps; ++it) {
+      const int s = it % S;
+      if (!mbar_wait(&full[s], (uint32_t)(it / S) & 1u)) {
+        atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint8_t* g = smem + s * stage;
+      const uint8_t* x = g + kWrJ * kWrRow;
+#pragma unroll
+      for (int kk = 0; kk < kWgPix / 16; ++kk) {
+        const uint64_t ad = sw64_mn_desc(g + kk * 1024, kWrRow, 512);
+        const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
+        umma(tmem, ad, sw64_mn_desc(x + kk * 1024, kWrRow, 512), id1, acc);
+        if (n2 > 0)
+          umma(tmem + 256, ad, sw64_mn_desc(x + 8 * kWrRow + kk * 1024, kWrRow, 512), id2, acc);
+      }
+      umma_commit(&empty[s]);
+    }
+    if (ok && steps > 0) umma_commit(accum);
+  }
+  __syncwarp();
+  const bool have = steps > 0 && __syncthreads_and(mbar_wait(accum, 0) ? 1 : 0) != 0;
+  if (steps > 0 && !have && threadIdx.x == 0) atomicCAS(&g_cnn_err, 0, MCA_ERR_TIMEOUT);
+  if (have || steps == 0) {
+    tc_fence_after();
+    float* stg = reinterpret_cast<float*>(smem);       // [j][ci][co]
+    const size_t T = (size_t)a.K * a.K;
+    for (int ky = 0; ky < a.K; ++ky) {
+      uint32_t v[32] = {};
+      if (have) tmem_ld32(tmem + (uint32_t)((warp + ky) * kC) + ((uint32_t)(warp * 32) << 16), v);
+#pragma unroll
+      for (int ci = 0; ci < kC; ++ci) stg[(warp * kC + ci) * kC + lane] = __uint_as_float(v[ci]);
+      __syncthreads();
+      float* dst = a.part + ((size_t)chunk * T + (size_t)ky * a.K + kx) * kC * kC;
+      for (int e = threadIdx.x; e < kC * kC; e += 128)
+        dst[e] = (stg[e] + stg[kC * kC + e]) + (stg[2 * kC * kC + e] + stg[3 * kC * kC + e]);
+      __syncthreads();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+  }
+}
+
 // gw[co][ci][t] = sum over chunks of part[chunk][t][ci][co] (fixed order), co < cout,
 // ci < cin: the master weight layout [cout][cin][K][K].
 __global__ void k_wgrad_reduce(const float* __restrict__ part, int nchunk, int T, int cin,
@@ -450,13 +937,21 @@ __global__ void k_bias_grad_part(const __nv_bfloat16* __restrict__ gz, size_t np
   }
 }
 
-__global__ void k_bias_grad_finish(const float* __restrict__ part, int nb, int cout,
-                                   float* __restrict__ gb) {
-  const int c = threadIdx.x;
-  if (c < cout) {
-    float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * kC + c];
-    gb[c] = s;
+// gb[c] from the nb blocks' sums: 32 x 32 threads, thread (g, c) sums the blocks g, g + 32,
+// ..., then one warp adds the 32 sums in order (one thread per channel over 4096 blocks took
+// 92 us).
+__global__ void __launch_bounds__(1024)
+k_bias_grad_finish(const float* __restrict__ part, int nb, int cout, float* __restrict__ gb) {
+  __shared__ float red[32][kC];
+  const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+  float s = 0.f;
+  for (int b = g; b < nb; b += 32) s += part[(size_t)b * kC + c];
+  red[g][c] = s;
+  __syncthreads();
+  if (g == 0 && c < cout) {
+    float t = 0.f;
+    for (int q = 0; q < 32; ++q) t += red[q][c];
+    gb[c] = t;
   }
 }
 
@@ -617,6 +1112,12 @@ cudaError_t configure() {
       e = cudaFuncSetAttribute(k_conv_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                227 * 1024);
     if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_conv_taps, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               227 * 1024);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_wgrad_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               227 * 1024);
+    if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_conv_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                WgLayout::SMEM);
     g_cfg_err = e;
@@ -660,6 +1161,33 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     set_last_cuda_error(e, "mca_cnn_conv configure", __FILE__, __LINE__);
     return MCA_ERR_CUDA;
   }
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  TapPlan tp{};
+  if (cout_mma == 32 && tap_plan(ksize, dilation, w, tp)) {
+    CUtensorMap tmW;
+    if ((reinterpret_cast<uintptr_t>(x) & 15) != 0 ||
+        !tc::make_map_taps(&tmW, wt, ksize, kC, kTapM)) {
+      set_error_message("mca_cnn_conv: tensor map encoding failed");
+      return MCA_ERR_UNSUPPORTED;
+    }
+    TapArgs a{};
+    a.H = h; a.W = w; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
+    a.xt = (w + tp.P - 1) / tp.P;
+    a.cout = cout; a.bias = bias; a.act = act; a.backward = backward;
+    a.yprev = reinterpret_cast<const __nv_bfloat16*>(y_prev);
+    a.out = reinterpret_cast<__nv_bfloat16*>(out);
+    a.out32 = out32;
+    a.x = reinterpret_cast<const __nv_bfloat16*>(x);
+    a.plan = tp;
+    a.tiles = n * h * a.xt;            // (n h w < 2^31)
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return launch_status("mca_cnn_conv device");
+    k_conv_taps<<<a.tiles < sms ? a.tiles : sms, kTapThreads, tp.smem, s>>>(tmW, a);
+    count_launches(1);
+    return launch_status("mca_cnn_conv launch");
+  }
   const ConvPlan plan = (cout_mma == 32) ? conv_plan<32>(ksize, dilation)
                                          : conv_plan<16>(ksize, dilation);
   if (plan.stages < 2 || plan.smem > 227 * 1024) {
@@ -679,7 +1207,6 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
   a.yprev = reinterpret_cast<const __nv_bfloat16*>(y_prev);
   a.out = reinterpret_cast<__nv_bfloat16*>(out);
   a.out32 = out32;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   dim3 grid((w + kPix - 1) / kPix, h, n);
   if (cout_mma == 32)
     k_conv_tc<32><<<grid, 128, plan.smem, s>>>(tmX, tmW, a);
@@ -716,24 +1243,46 @@ int mca_cnn_conv_wgrad(const uint16_t* x, const uint16_t* gz, int32_t n, int32_t
     return MCA_ERR_UNSUPPORTED;
   }
   const int T = ksize * ksize;
-  WgArgs a{};
-  a.N = n; a.H = h; a.W = w; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
-  a.rows_total = n * h;
-  a.nxc = (w + kWgPix - 1) / kWgPix;
-  a.part = scratch;
-  const int nchunk = (a.rows_total + kWgRows - 1) / kWgRows;
+  // partial sums: the scratch holds one set per kWgRows image rows
+  const int nmax = (int)(((int64_t)n * h + kWgRows - 1) / kWgRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  dim3 grid((T + kWgTaps - 1) / kWgTaps, nchunk);
-  k_conv_wgrad_tc<<<grid, 128, WgLayout::SMEM, s>>>(tmX, tmG, a);
+  int nchunk;
+  if (ksize >= 5 && ksize <= kWrMaxK) {
+    WrArgs a{};
+    a.H = h; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
+    const int rem = h % (kWrJ * dilation);
+    a.blocks = h / (kWrJ * dilation) * dilation + (rem < dilation ? rem : dilation);
+    a.nxc = (w + kWgPix - 1) / kWgPix;
+    a.items = n * a.blocks * a.nxc;
+    a.part = scratch;
+    // small images: two CTAs' shares per SM (one CTA resides at a time)
+    nchunk = (a.items + kWrItems - 1) / kWrItems;
+    if (nchunk < 2 * 152 / ksize) nchunk = 2 * 152 / ksize;
+    if (nchunk > nmax) nchunk = nmax;
+    if (nchunk > a.items) nchunk = a.items;
+    const int stage = (ksize + 2 * kWrJ - 1) * kWrRow;
+    a.stages = kWrStages * stage <= 224 * 1024 ? kWrStages : 2;
+    const int smem = a.stages * stage + 512 + 1024;
+    k_wgrad_rows<<<dim3(ksize, nchunk), 128, smem, s>>>(tmX, tmG, a);
+  } else {
+    WgArgs a{};
+    a.N = n; a.H = h; a.W = w; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
+    a.rows_total = n * h;
+    a.nxc = (w + kWgPix - 1) / kWgPix;
+    a.part = scratch;
+    nchunk = nmax;
+    dim3 grid((T + kWgTaps - 1) / kWgTaps, nchunk);
+    k_conv_wgrad_tc<<<grid, 128, WgLayout::SMEM, s>>>(tmX, tmG, a);
+  }
   k_wgrad_reduce<<<grid1d((size_t)T * cin * cout, 256), 256, 0, s>>>(scratch, nchunk, T, cin,
                                                                       cout, gw);
   count_launches(2);
   if (gb) {
     const size_t npix = (size_t)n * h * w;
-    const int nb = grid1d(npix, 256);
-    float* pb = scratch + (size_t)nchunk * T * kC * kC;
+    const int nb = std::min(grid1d(npix, 256), 8 * 152);
+    float* pb = scratch + (size_t)nmax * T * kC * kC;
     k_bias_grad_part<<<nb, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16*>(gz), npix, cout, pb);
-    k_bias_grad_finish<<<1, 32, 0, s>>>(pb, nb, cout, gb);
+    k_bias_grad_finish<<<1, 1024, 0, s>>>(pb, nb, cout, gb);
     count_launches(2);
   }
   return launch_status("mca_cnn_conv_wgrad launch");

@@ -908,6 +908,19 @@ bool make_map_nhwc32_k8(CUtensorMap* map, const void* base, uint64_t W, uint64_t
   return r == CUDA_SUCCESS;
 }
 
+bool make_map_taps(CUtensorMap* map, const void* base, uint32_t K, uint32_t rows, uint32_t taps) {
+  if (!encode_available()) return false;
+  cuuint64_t gdim[4] = {32, rows, K, K};
+  cuuint64_t gstride[3] = {64, 64 * (cuuint64_t)rows, 64 * (cuuint64_t)rows * K};
+  cuuint32_t box[4] = {32, rows, taps, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = g_encode.load()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base),
+                               gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 cudaError_t gemm(int bn, int split, int epi, const CUtensorMap& a, const CUtensorMap& al,
                  const CUtensorMap& bm, const CUtensorMap& bml, const GemmEpi& ep, int B,
                  cudaStream_t s) {

@@ -55,6 +55,9 @@ bool make_map_nhwc32(CUtensorMap* map, const void* base, uint64_t W, uint64_t H,
 // box_px consecutive 16-byte rows (one K chunk of a K-major operand without swizzling)
 bool make_map_nhwc32_k8(CUtensorMap* map, const void* base, uint64_t W, uint64_t H, uint64_t N,
                         uint32_t box_px);
+// 4-D map over weight tiles [ky][kx][rows][32] of a K x K kernel, box = `taps` neighbouring
+// taps of one kernel row (64-byte swizzle; taps beyond the row read zero)
+bool make_map_taps(CUtensorMap* map, const void* base, uint32_t K, uint32_t rows, uint32_t taps);
 cudaError_t gemm(int bn, int split, int epi, const CUtensorMap& a, const CUtensorMap& al,
                  const CUtensorMap& bm, const CUtensorMap& bml, const GemmEpi& ep, int B,
                  cudaStream_t s);

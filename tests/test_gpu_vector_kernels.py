@@ -146,3 +146,57 @@ def test_fp64_preconditioner_of_part_of_a_batch(m, n, nvec):
             zs.append(torch.empty_like(rd))
             s.precond_apply(np.full(nvec, 2.1e-5), rd, zs[-1])
     assert torch.equal(zs[0], zs[1])
+
+
+@pytest.mark.parametrize("K,d,H,W", [(5, 1, 3, 70), (11, 1, 13, 130), (11, 2, 5, 40),
+                                     (11, 8, 40, 260), (11, 32, 70, 150), (7, 3, 9, 16),
+                                     (13, 1, 20, 65), (15, 1, 18, 64), (9, 43, 50, 100)])
+def test_convolution_forms(K, d, H, W):
+    """The convolutions' and the weight gradient's row forms and the forms they fall back to
+    (kernels of 15, dilations whose four taps do not fit): odd rows, rows without a partner, tiles
+    cut by the image, taps beyond the kernel row.  FP32 accumulation of exact BF16 products:
+    1e-5 of the summed term magnitudes (forward, backward data, weights), BF16 outputs within
+    2^-8 of the value besides."""
+    lib = mca.load()
+    N, C = 2, 32
+    g = torch.Generator(device=DEV).manual_seed(K * H + d)
+
+    def rnd(*shape):
+        return torch.randn(*shape, generator=g, device=DEV).to(torch.bfloat16)
+
+    x, gz = rnd(N, H, W, C), rnd(N, H, W, C)
+    w = (rnd(C, C, K, K).float() / (C * K * K) ** 0.5).to(torch.bfloat16).float()
+    bias = torch.randn(C, generator=g, device=DEV)
+    wf = torch.empty(K * K, C, C, dtype=torch.int16, device=DEV)
+    wb = torch.empty_like(wf)
+    out, gx = torch.empty_like(x), torch.empty_like(x)
+    gw, gb = torch.empty_like(w), torch.empty_like(bias)
+    scratch = torch.empty(int(lib.mca_cnn_wgrad_scratch(N, H, W, K)), device=DEV)
+    p = [t.data_ptr() for t in (x, gz, wf, wb, bias, out, gx, gw, gb, scratch)]
+    assert lib.mca_cnn_prep_weights(w.data_ptr(), C, C, K, C, p[2], p[3], None) == 0
+    assert lib.mca_cnn_conv(p[0], N, H, W, p[2], K, d, C, C, p[4], 1, 0, None, p[5], None, None) == 0
+    assert lib.mca_cnn_conv(p[1], N, H, W, p[3], K, d, C, C, None, 1, 1, p[0], p[6], None, None) == 0
+    assert lib.mca_cnn_conv_wgrad(p[0], p[1], N, H, W, K, d, C, C, p[9], p[7], p[8], None) == 0
+    assert lib.mca_cnn_check(None) == 0
+
+    def ref(xv, wv, gzv):
+        xv = xv.double().permute(0, 3, 1, 2).cpu().requires_grad_(True)
+        wv = wv.double().cpu().requires_grad_(True)
+        y = torch.nn.functional.conv2d(xv, wv, padding=d * (K // 2), dilation=d)
+        y.backward(gzv.double().permute(0, 3, 1, 2).cpu())
+        return [t.detach() for t in (y, xv.grad, wv.grad)]
+
+    y, dx, dw = ref(x, w, gz)
+    ys, dxs, dws = ref(x.abs(), w.abs(), gz.abs())
+    z = y + bias.double().cpu()[None, :, None, None]
+    zs = ys + bias.double().cpu().abs()[None, :, None, None]
+    z = torch.where(z > 0, z, 0.1 * z)
+    got = out.double().permute(0, 3, 1, 2).cpu()
+    assert bool(((got - z).abs() <= 2.0 ** -8 * z.abs() + 1e-5 * zs).all())
+    xc = x.double().permute(0, 3, 1, 2).cpu()
+    dx = torch.where(xc > 0, dx, 0.1 * dx)
+    got = gx.double().permute(0, 3, 1, 2).cpu()
+    assert bool(((got - dx).abs() <= 2.0 ** -8 * dx.abs() + 1e-5 * dxs).all())
+    assert bool(((gw.double().cpu() - dw).abs() <= 1e-5 * dws).all())
+    gs = gz.double().sum(dim=(0, 1, 2)).cpu()
+    assert bool(((gb.double().cpu() - gs).abs() <= 1e-5 * gz.double().abs().sum(dim=(0, 1, 2)).cpu()).all())
