@@ -16,14 +16,14 @@
 // power of two and cut into 8 slices of signed 7-bit digits,
 //   x = 2^(e + 2) sum_s a_s 128^-(s + 1),   |a_s| <= 64,
 // which BF16 holds exactly; products of digits are integers of at most 2^12, so that the FP32
-// accumulators of the tensor core hold their sums over K <= 4096 exactly; and the sums of
-// equal weight d = s + t, d = 0 .. 7 (36 of the 64 slice products) are added to one FP64
-// result, rounded once.  What is dropped lies below 2^-54 of (row maximum) x (column
+// accumulators of the tensor core hold exactly what the up to 8 slice products of one weight
+// d = s + t sum over K <= 512 (8 x 512 x 2^12 = 2^24); and the sums of weights 0 .. 7 (36 of
+// the 64 slice products) are joined to one FP64 result per 512 of K, rounded once.  What is dropped lies below 2^-54 of (row maximum) x (column
 // maximum) per product, where a chain of FMAs rounds at 2^-53 of its partial sums at every
 // step: the apply's error against quadruple precision is half that of the FMA chain's
 // (256 x 256: 5.8e-16 against 1.2e-15).
 // One apply (four transforms), against the FMA kernel: 512 x 512, 4 vectors 520 us (8300),
-// 1024 x 1024 770 us (16500), 64 x 64 135 us (324), 16 x 16 108 us (126).
+// 1024 x 1024 933 us (16500), 64 x 64 135 us (324), 16 x 16 110 us (126).
 #include <cuda.h>
 
 #include <algorithm>
@@ -50,7 +50,7 @@ constexpr int kOzStage = kSlices * (kOzA + kOzB);                  // 96 KB
 constexpr int kOzStages = 2;
 constexpr int kOzBar = kOzStages * kOzStage;
 constexpr int kOzSmem = kOzBar + 256 + 1024;
-constexpr int kOzKMax = 4096;     // largest K summed in one FP32 accumulator
+constexpr int kOzKMax = 512;      // largest K whose 8 products per weight FP32 sums hold exactly
 constexpr int kBadRow = 0x7FFFFFFF;   // exponent of a row with an infinity or a NaN
 constexpr int kZeroRow = -0x7FFFFFFF; // and of a row of zeros
 

@@ -133,6 +133,29 @@ def test_fp64_preconditioner_in_slices(m, n):
         assert np.linalg.norm(P @ z[v] - r[v]) <= 1e-9 * size * np.linalg.norm(z[v])
 
 
+@pytest.mark.parametrize("n", [512, 4000])
+def test_fp64_slices_of_coherent_rows(n):
+    """A constant right-hand side against the nearly constant lowest mode: the slice products of
+    a weight all have one sign and sum beyond 2^24 unless K is cut.  Extended-precision sums
+    with the handle's own eigenpairs; rounding stays within 4 transforms x n ulps."""
+    cb = mi.make_crossbar(1, n, 4)
+    weak = dict(g_src=1e-12, g_term_top_right=1e-12)
+    with mca.Solver(mca.default_params(1, n, precision=mca.PREC_FP64, max_batch=1, **weak),
+                    cb.gmap) as s:
+        mu, qr, nu, _ = s.eigenpairs()
+        a = 2.1e-5
+        z = torch.empty(1, 2 * n, dtype=torch.float64, device=DEV)
+        s.precond_apply(np.array([a]), torch.full_like(z, 63.4921875 / 32), z)
+    ld = np.longdouble
+    x = qr.astype(ld).T @ np.full(n, 63.4921875 / 32, ld)
+    mu, nu0, a = mu.astype(ld), ld(nu[0]), ld(a)
+    det = mu * nu0 + mu * a + nu0 * a
+    ref = np.concatenate([qr.astype(ld) @ ((nu0 + a + a) * x / det),
+                          qr.astype(ld) @ ((mu + a + a) * x / det)])
+    err = np.abs(z.cpu().numpy()[0] - ref).max() / np.abs(ref).max()
+    assert err <= 4 * n * 2.0 ** -53
+
+
 @pytest.mark.parametrize("m,n,nvec", [(5, 130, 1), (129, 65, 2)])
 def test_fp64_preconditioner_of_part_of_a_batch(m, n, nvec):
     """Fewer vectors than the handle holds: the same values as in a handle made for them."""
