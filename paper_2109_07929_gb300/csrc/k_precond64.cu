@@ -18,8 +18,9 @@
 // which BF16 holds exactly; products of digits are integers of at most 2^12, so that the FP32
 // accumulators of the tensor core hold exactly what the up to 8 slice products of one weight
 // d = s + t sum over K <= 512 (8 x 512 x 2^12 = 2^24); and the sums of weights 0 .. 7 (36 of
-// the 64 slice products) are joined to one FP64 result per 512 of K, rounded once.  What is dropped lies below 2^-54 of (row maximum) x (column
-// maximum) per product, where a chain of FMAs rounds at 2^-53 of its partial sums at every
+// the 64 slice products) are joined to one FP64 result per 512 of K, rounded once.  What is
+// dropped lies below 2^-54 of (row maximum) x (column maximum) per product, where a chain of
+// FMAs rounds at 2^-53 of its partial sums at every
 // step: the apply's error against quadruple precision is half that of the FMA chain's
 // (256 x 256: 5.8e-16 against 1.2e-15).
 // One apply (four transforms), against the FMA kernel: 512 x 512, 4 vectors 520 us (8300),
