@@ -760,14 +760,17 @@ k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // share of the images' row blocks; the epilogue adds the four diagonals and writes one
 // partial sum per CTA.  Rows beyond the image read zero (a NaN in x reaches, where the row
 // blocks do not divide H, taps whose own gradient rows all lie outside).
-// Bound: L2 reads and MMA issue.  32 images of 256 x 256, 11 x 11, dilation 4: 2583 us, now
-// 660.
+// Bound: L2 reads and MMA issue.  32 images of 256 x 256, 11 x 11, dilation 4, with the sums
+// behind it: 2779 us per call, now 685.
 constexpr int kWrJ = 4;                                 // gradient rows per CTA step
 constexpr int kWrRow = kWgPix * kC * 2;                 // 64 pixels of a row: 4 KB
 constexpr int kWrMaxK = 512 / kC - (kWrJ - 1);          // 13
 constexpr int kWrStages = 3;                            // (2 where 3 do not fit: K = 13)
-// Row-block chunks per partial sum: 256 MMA steps per accumulator, as many as the other form
-// takes on 256-pixel rows (the tensor core's FP32 sums lose about a rounding per step)
+// Row-block chunks per partial sum, at most: 256 MMA steps per accumulator, as many as the
+// other form takes on 256-pixel rows, and on narrower rows its number there, kWgRows rows of
+// chunks (the tensor core's FP32 sums lose about a rounding per step.  32 images of 92 x 92,
+// dilation 8, 11 x 11: relative error against FP64 2.0e-6 with up to 64, 1.1e-6 with up to
+// 32; the other form's 1.4e-6)
 constexpr int kWrItems = 64;
 
 struct WrArgs {
@@ -1125,6 +1128,13 @@ cudaError_t configure() {
   return g_cfg_err;
 }
 
+cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e
+                          : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 int launch_status(const char* what) {
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1180,10 +1190,11 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     a.x = reinterpret_cast<const __nv_bfloat16*>(x);
     a.plan = tp;
     a.tiles = n * h * a.xt;            // (n h w < 2^31)
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return launch_status("mca_cnn_conv device");
+    int sms = 0;
+    if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
+      set_last_cuda_error(e, "mca_cnn_conv device", __FILE__, __LINE__);
+      return MCA_ERR_CUDA;
+    }
     k_conv_taps<<<a.tiles < sms ? a.tiles : sms, kTapThreads, tp.smem, s>>>(tmW, a);
     count_launches(1);
     return launch_status("mca_cnn_conv launch");
@@ -1255,9 +1266,17 @@ int mca_cnn_conv_wgrad(const uint16_t* x, const uint16_t* gz, int32_t n, int32_t
     a.nxc = (w + kWgPix - 1) / kWgPix;
     a.items = n * a.blocks * a.nxc;
     a.part = scratch;
-    // small images: two CTAs' shares per SM (one CTA resides at a time)
-    nchunk = (a.items + kWrItems - 1) / kWrItems;
-    if (nchunk < 2 * 152 / ksize) nchunk = 2 * 152 / ksize;
+    int sms = 0;
+    if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
+      set_last_cuda_error(e, "mca_cnn_conv_wgrad device", __FILE__, __LINE__);
+      return MCA_ERR_CUDA;
+    }
+    const int most = std::min(kWrItems, kWgRows * a.nxc);
+    nchunk = (a.items + most - 1) / most;
+    // whole waves of CTAs (one resides per SM), two at least: 11 images of 187 x 187, dilation
+    // 8, 182 us per call with 33 chunks (2.4 waves), 158 with 41; 32 of 256 x 256, 717 and 685
+    const int waves = std::max(2, (ksize * nchunk + sms - 1) / sms);
+    nchunk = std::max(nchunk, waves * sms / ksize);
     if (nchunk > nmax) nchunk = nmax;
     if (nchunk > a.items) nchunk = a.items;
     const int stage = (ksize + 2 * kWrJ - 1) * kWrRow;
