@@ -758,8 +758,9 @@ k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // whose blocks i = j + ky are the four rows' parts of tap (ky, kx): 4 K of 4 (K + 3) blocks
 // are used, and 72 KB per 64 pixels feed 900 clocks of MMAs (K = 11).  D accumulates over a
 // share of the images' row blocks; the epilogue adds the four diagonals and writes one
-// partial sum per CTA.  Rows beyond the image read zero (a NaN in x reaches, where the row
-// blocks do not divide H, taps whose own gradient rows all lie outside).
+// partial sum per CTA.  Gradient rows beyond the image, where the row blocks do not divide H,
+// are kept out of D by the MMA's lane mask and not only by their zeros, which an infinity or a
+// NaN in x would turn into NaN; D starts from zeros, so that every MMA can have a mask.
 // Bound: L2 reads and MMA issue.  32 images of 256 x 256, 11 x 11, dilation 4, with the sums
 // behind it: 2779 us per call, now 685.
 constexpr int kWrJ = 4;                                 // gradient rows per CTA step
@@ -815,6 +816,20 @@ k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  for (int c = 0; c < rows; ++c)
+    tmem_zero32(tmem + (uint32_t)(c * kC) + ((uint32_t)(warp * 32) << 16));
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  // first gradient row of a row block, and the image n and pixel x0 of an item
+  auto first_row = [&](int item, int& n, int& x0) {
+    const int rb = item / a.nxc;
+    x0 = (item - rb * a.nxc) * kWgPix;
+    n = rb / a.blocks;
+    const int blk = rb - n * a.blocks;
+    return blk / a.d * kWrJ * a.d + blk % a.d;
+  };
   if (threadIdx.x == 0) {
     for (int it = 0; it < steps; ++it) {
       const int s = it % S;
@@ -824,10 +839,8 @@ k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
       }
       uint8_t* st = smem + s * stage;
       mbar_expect_tx(&full[s], (uint32_t)stage);
-      const int item = it0 + it;
-      const int xc = item % a.nxc, rb = item / a.nxc;
-      const int n = rb / a.blocks, blk = rb - n * a.blocks;
-      const int y = blk / a.d * kWrJ * a.d + blk % a.d, x0 = xc * kWgPix;
+      int n, x0;
+      const int y = first_row(it0 + it, n, x0);
       for (int j = 0; j < kWrJ; ++j)
         tma_load_4d(st + j * kWrRow, &tmG, 0, x0, y + j * a.d, n, &full[s]);
       for (int i = 0; i < rows; ++i)
@@ -848,13 +861,18 @@ k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
       tc_fence_after();
       const uint8_t* g = smem + s * stage;
       const uint8_t* x = g + kWrJ * kWrRow;
+      int n, x0;
+      const int y = first_row(it0 + it, n, x0);
+      uint32_t off[kWrJ];
+#pragma unroll
+      for (int j = 0; j < kWrJ; ++j) off[j] = (y + j * a.d < a.H) ? 0u : 0xffffffffu;
 #pragma unroll
       for (int kk = 0; kk < kWgPix / 16; ++kk) {
         const uint64_t ad = sw64_mn_desc(g + kk * 1024, kWrRow, 512);
-        const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
-        umma(tmem, ad, sw64_mn_desc(x + kk * 1024, kWrRow, 512), id1, acc);
+        umma_lanes(tmem, ad, sw64_mn_desc(x + kk * 1024, kWrRow, 512), id1, 1u, off);
         if (n2 > 0)
-          umma(tmem + 256, ad, sw64_mn_desc(x + 8 * kWrRow + kk * 1024, kWrRow, 512), id2, acc);
+          umma_lanes(tmem + 256, ad, sw64_mn_desc(x + 8 * kWrRow + kk * 1024, kWrRow, 512), id2,
+                     1u, off);
       }
       umma_commit(&empty[s]);
     }

@@ -43,3 +43,38 @@ def test_weight_gradient_partial_sums_are_short(K, d, N, H, W):
     blocks = whole * d + min(rest, d)            # blocks of four gradient rows per image
     steps = 4 * -(-N * blocks * chunks // written)
     assert steps <= 4 * min(64, 16 * chunks)
+
+
+def _reach(t):
+    """0 finite, 1 infinity, 2 minus infinity, 3 NaN."""
+    t = t.double().cpu()
+    return (torch.isposinf(t).int() + 2 * torch.isneginf(t).int() + 3 * torch.isnan(t).int())
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("K,d,H,W", [(5, 1, 9, 64), (7, 2, 30, 128), (11, 4, 70, 64),
+                                     (13, 1, 21, 64), (11, 32, 50, 64)])
+def test_weight_gradient_reach_of_infinities(K, d, H, W, value):
+    """An infinity or a NaN in x reaches the taps that multiply it with a pixel of the gradient,
+    and no others: rows of the images past the last gradient row have none (widths are whole
+    chunks of 64 pixels, so that no pixel past the row's end takes part).  gz > 0, so the
+    reached taps are the value itself."""
+    N = 2
+    g = torch.Generator(device=DEV).manual_seed(K * H)
+    x, gz = ((torch.rand((N, H, W, C), generator=g, device=DEV) + 0.5).to(torch.bfloat16)
+             for _ in range(2))
+    spots = [(0, 0, 0, 3), (0, H - 1, W - 1, 5), (1, H // 2, W // 3, 7)]
+    for n, y, xx, ci in spots:
+        x[n, y, xx, ci] = value
+    gw, gb, _ = _weight_gradient(x, gz, K, d)
+    want = torch.zeros(C, C, K, K, dtype=torch.int32)
+    kind = 3 if value != value else 1
+    r = K // 2
+    for n, y, xx, ci in spots:
+        for ky in range(K):
+            for kx in range(K):
+                py, px = y - (ky - r) * d, xx - (kx - r) * d
+                if 0 <= py < H and 0 <= px < W:
+                    want[:, ci, ky, kx] = kind
+    assert torch.equal(_reach(gw), want)
+    assert int(_reach(gb).sum()) == 0
