@@ -283,9 +283,11 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
 // pixel rows without swizzle: any start), so that all groups add to one accumulator, and
 //   out[co][x0 + p] = sum_q D_q[co][p + q d]
 // is left to the epilogue: N = P + 3 d columns for P pixels.  Taps beyond the kernel row read
-// as zero weights (TMA bounds; where K is no multiple of 4, an infinity or NaN in x therefore
-// reaches up to 3 output pixels more per row than its window); input rows outside the image
-// are left out.
+// as zero weights (TMA bounds), which an infinity or a NaN up to 3 d pixels outside a window turns
+// into NaN: an output that comes out NaN is summed again over its own window (window_sum).
+// Keeping those taps out by the MMA's lane mask took 806 us for the 32 images below, halving the
+// weights of an overlapping last group in shared memory 1140.  Input rows outside the image are
+// left out.
 // One persistent CTA per SM walks the tiles (P pixels of one image row): per stage, warp 0
 // brings in a kernel row's weights (TMA) and 8 warps its input row, warp 1 issues 2 G MMAs of
 // 128 x N x 16 into one of two accumulators, and 8 warps drain the other one, 64 pixels at a
@@ -344,7 +346,7 @@ struct TapArgs {
   int H, W, K, d, r;
   int xt, tiles;                       // tiles per image row and in all
   int cout;
-  const __nv_bfloat16* x;
+  const __nv_bfloat16 *x, *w;          // w: [ky][kx][co][ci]
   const float* bias;
   int act, backward;
   const __nv_bfloat16* yprev;
@@ -352,6 +354,28 @@ struct TapArgs {
   float* out32;
   TapPlan plan;
 };
+
+// The convolution's sum of channel co at pixel (y, x) of image n, without bias, term by term: for
+// outputs in whose accumulators an infinity or a NaN has been.  Ends at a NaN.
+__device__ __forceinline__ float window_sum(const TapArgs& a, int n, int y, int x, int co) {
+  float s = 0.f;
+#pragma unroll 1
+  for (int ky = 0; ky < a.K; ++ky) {
+    const int yy = y + (ky - a.r) * a.d;
+    const bool row = yy >= 0 && yy < a.H;
+#pragma unroll 1
+    for (int kx = 0; kx < a.K && s == s; ++kx) {
+      const int xx = x + (kx - a.r) * a.d;
+      const bool in = row && xx >= 0 && xx < a.W;
+      const __nv_bfloat16* px = a.x + (in ? (((size_t)n * a.H + yy) * a.W + xx) * kC : 0);
+      const __nv_bfloat16* wt = a.w + ((size_t)(ky * a.K + kx) * kC + co) * kC;
+#pragma unroll 1
+      for (int ci = 0; ci < kC; ++ci)
+        s = fmaf(in ? __bfloat162float(px[ci]) : 0.f, __bfloat162float(wt[ci]), s);
+    }
+  }
+  return s;
+}
 
 // 16 bytes to shared memory, zeros when !ok (src must be readable memory either way)
 __device__ __forceinline__ void copy16_async(uint32_t dst, const void* src, bool ok) {
@@ -367,7 +391,7 @@ __device__ __forceinline__ void copies_wait() {
 }
 
 __global__ void __launch_bounds__(kTapThreads, 1)
-k_conv_taps(const __grid_constant__ CUtensorMap tmW, TapArgs a) {
+k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ TapArgs a) {
   const TapPlan& P = a.plan;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -568,6 +592,15 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, TapArgs a) {
             const float4 u = src[0], w = src[1];
             o[0] += u.x; o[1] += u.y; o[2] += u.z; o[3] += u.w;
             o[4] += w.x; o[5] += w.y; o[6] += w.z; o[7] += w.w;
+          }
+          const float any = ((o[0] + o[1]) + (o[2] + o[3])) + ((o[4] + o[5]) + (o[6] + o[7]));
+          if (any != any) {
+#pragma unroll 1
+            for (int c = 0; c < 8; ++c) {
+              const float sum = window_sum(a, n, y, x, c8 + c);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) o[k] = (k == c) ? sum : o[k];
+            }
           }
           const __nv_bfloat16* ypb = reinterpret_cast<const __nv_bfloat16*>(&yp);
 #pragma unroll
@@ -1206,6 +1239,7 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     a.out = reinterpret_cast<__nv_bfloat16*>(out);
     a.out32 = out32;
     a.x = reinterpret_cast<const __nv_bfloat16*>(x);
+    a.w = reinterpret_cast<const __nv_bfloat16*>(wt);
     a.plan = tp;
     a.tiles = n * h * a.xt;            // (n h w < 2^31)
     int sms = 0;

@@ -78,3 +78,50 @@ def test_weight_gradient_reach_of_infinities(K, d, H, W, value):
                     want[:, ci, ky, kx] = kind
     assert torch.equal(_reach(gw), want)
     assert int(_reach(gb).sum()) == 0
+
+
+def _convolve(x, w, d, bias=None, backward_of=None):
+    """The layer's forward convolution, or with backward_of = its input the backward data one
+    of the output gradient x."""
+    lib = mca.load()
+    N, H, W, _ = x.shape
+    K = w.shape[-1]
+    wf = torch.empty(K * K, C, C, dtype=torch.int16, device=DEV)
+    wb = torch.empty_like(wf)
+    assert lib.mca_cnn_prep_weights(w.data_ptr(), C, C, K, C, wf.data_ptr(), wb.data_ptr(),
+                                    None) == 0
+    out = torch.empty_like(x)
+    if backward_of is None:
+        rc = lib.mca_cnn_conv(x.data_ptr(), N, H, W, wf.data_ptr(), K, d, C, C, bias.data_ptr(), 0,
+                              0, None, out.data_ptr(), None, None)
+    else:
+        rc = lib.mca_cnn_conv(x.data_ptr(), N, H, W, wb.data_ptr(), K, d, C, C, None, 1, 1,
+                              backward_of.data_ptr(), out.data_ptr(), None, None)
+    assert rc == 0 and lib.mca_cnn_check(None) == 0
+    return out
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("K,d,H,W", [(5, 1, 9, 70), (7, 2, 30, 50), (9, 1, 17, 64), (11, 4, 70, 90),
+                                     (11, 32, 70, 150), (13, 1, 20, 65), (15, 1, 18, 64)])
+def test_convolution_reach_of_infinities(K, d, H, W, value):
+    """An infinity or a NaN in a pixel reaches the outputs whose window holds it, and no others,
+    forward and backward (weights > 0: the reached outputs are the value itself)."""
+    N = 2
+    g = torch.Generator(device=DEV).manual_seed(K * H)
+    x = (torch.rand((N, H, W, C), generator=g, device=DEV) + 0.5).to(torch.bfloat16)
+    below = x.clone()
+    w = torch.rand((C, C, K, K), generator=g, device=DEV) + 0.5
+    spots = [(0, 0, 0, 3), (0, H - 1, W - 1, 5), (1, H // 2, W // 3, 7)]
+    for n, y, xx, ci in spots:
+        x[n, y, xx, ci] = value
+    want = torch.zeros(N, H, W, C, dtype=torch.int32)
+    reach = [(i - K // 2) * d for i in range(K)]
+    for n, y, xx, _ in spots:
+        rows = [y + i for i in reach if 0 <= y + i < H]
+        cols = [xx + i for i in reach if 0 <= xx + i < W]
+        for yy in rows:
+            want[n, yy, cols] = 3 if value != value else 1
+    bias = torch.zeros(C, device=DEV)
+    assert torch.equal(_reach(_convolve(x, w, d, bias)), want)
+    assert torch.equal(_reach(_convolve(x, w, d, backward_of=below)), want)
