@@ -287,14 +287,16 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
 // into NaN: an output that comes out NaN is summed again over its own window (window_sum).
 // Keeping those taps out by the MMA's lane mask took 806 us for the 32 images below, halving the
 // weights of an overlapping last group in shared memory 1140.  Input rows outside the image are
-// left out.
+// left out; as zeros they would still turn weights that are no numbers into NaN, so the drain
+// looks at the weights of those kernel rows (once per CTA, while it waits) and sums the outputs
+// of such channels again too.
 // One persistent CTA per SM walks the tiles (P pixels of one image row): per stage, warp 0
 // brings in a kernel row's weights (TMA) and 8 warps its input row, warp 1 issues 2 G MMAs of
 // 128 x N x 16 into one of two accumulators, and 8 warps drain the other one, 64 pixels at a
 // time.  The input rows go through 16-byte asynchronous copies: a TMA box of one 8-channel
 // plane consists of 16-byte rows, and 700 of those per stage took three times its MMAs.
 // Bound: the input rows' copies and the drain, each about 1200 clocks per stage against 430
-// of MMAs.  32 images of 256 x 256, 11 x 11, dilation 4: 1495 us, now 760 (one CTA per tile
+// of MMAs.  32 images of 256 x 256, 11 x 11, dilation 4: 1495 us, now 775 (one CTA per tile
 // with the drain exposed: 1081; persistent with TMA input rows: 828).
 constexpr int kTapM = 4;               // taps per M tile
 constexpr int kTapPad = 36;            // floats per pixel of the epilogue's staging rows
@@ -404,6 +406,7 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ Tap
   uint64_t* tempty = tfull + 2;                      // [2] accumulator drained
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   volatile uint32_t& dead = tmem_slot[1];            // a drain warp's wait gave up
+  uint32_t* wbad = tmem_slot + 2;                    // channels without numbers per kernel row; any
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = a.d;
   // tile t: P pixels from x0 of row y of image n, and the kernel rows that meet the image
@@ -415,6 +418,7 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ Tap
     k0 = max(0, a.r - y / d);
     k1 = min(a.K - 1, a.r + (a.H - 1 - y) / d);
   };
+  if (threadIdx.x <= kMaxK) wbad[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     dead = 0;
     for (int s = 0; s < S; ++s) {
@@ -549,6 +553,41 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ Tap
     for (int c = 0; c < 8; ++c)
       bias[c] = (!a.backward && a.bias && c8 + c < a.cout) ? a.bias[c8 + c] : 0.f;
     const bool gate = a.backward && a.act && a.yprev;
+    // the weights of kernel rows outside the image of any of the CTA's tiles: [0, lo), [hi, K)
+    int lo = 0, hi = a.K;
+    for (int t = blockIdx.x + lane * gridDim.x; t < a.tiles; t += 32 * gridDim.x) {
+      int n, y, x0, k0, k1;
+      decode(t, n, y, x0, k0, k1);
+      lo = max(lo, k0);
+      hi = min(hi, k1 + 1);
+    }
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    hi = __reduce_min_sync(0xffffffffu, hi);
+    const int per_row = a.K * (kC * kC / 8);           // 16-byte pieces of a row's weights
+    const int skip = (hi - lo) * per_row, all = (a.K - (hi - lo)) * per_row;
+    constexpr int kLook = 8;                           // loads in flight per thread
+    for (int e0 = tid; e0 < all; e0 += kLook * kTapDrain) {
+      uint4 u[kLook];
+#pragma unroll
+      for (int q = 0; q < kLook; ++q) {
+        const int e = min(e0 + q * kTapDrain, all - 1);
+        u[q] = reinterpret_cast<const uint4*>(a.w)[e + (e >= lo * per_row ? skip : 0)];
+      }
+      uint32_t nan = 0;
+#pragma unroll
+      for (int q = 0; q < kLook; ++q) {
+        const uint32_t v[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if ((v[k] & 0x7F80u) == 0x7F80u || (v[k] & 0x7F800000u) == 0x7F800000u) nan |= 1u << q;
+      }
+      for (; nan != 0; nan &= nan - 1) {
+        int e = min(e0 + (__ffs(nan) - 1) * kTapDrain, all - 1);
+        e += (e >= lo * per_row) ? skip : 0;
+        atomicOr(&wbad[e / per_row], 1u << ((e >> 2) & (kC - 1)));
+        wbad[kMaxK] = 1;
+      }
+    }
     int tl = 0;
     for (int t = blockIdx.x; t < a.tiles; t += gridDim.x, ++tl) {
       int n, y, x0, k0, k1;
@@ -563,6 +602,9 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ Tap
       asm volatile("bar.sync 1, %0;" ::"n"(kTapDrain) : "memory");
       if (dead) break;                 // (all 8 warps: a wait that gave up)
       tc_fence_after();
+      uint32_t bad = 0;                // channels whose weights outside the image are no numbers
+      if (wbad[kMaxK])
+        for (int ky = 0; ky < a.K; ++ky) bad |= (ky < k0 || ky > k1) ? wbad[ky] : 0u;
       for (int p0 = 0; p0 < P.P; p0 += kTapChunk) {
         const int p = p0 + pl, x = x0 + p;
         const bool in = p < P.P && x < a.W;
@@ -594,7 +636,7 @@ k_conv_taps(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ Tap
             o[4] += w.x; o[5] += w.y; o[6] += w.z; o[7] += w.w;
           }
           const float any = ((o[0] + o[1]) + (o[2] + o[3])) + ((o[4] + o[5]) + (o[6] + o[7]));
-          if (any != any) {
+          if (any != any || ((bad >> c8) & 0xFFu) != 0) {
 #pragma unroll 1
             for (int c = 0; c < 8; ++c) {
               const float sum = window_sum(a, n, y, x, c8 + c);

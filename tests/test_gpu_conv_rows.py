@@ -125,3 +125,25 @@ def test_convolution_reach_of_infinities(K, d, H, W, value):
     bias = torch.zeros(C, device=DEV)
     assert torch.equal(_reach(_convolve(x, w, d, bias)), want)
     assert torch.equal(_reach(_convolve(x, w, d, backward_of=below)), want)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+@pytest.mark.parametrize("K,d,H,W", [(5, 1, 9, 70), (7, 2, 30, 50), (11, 4, 70, 90), (11, 4, 5, 40),
+                                     (13, 1, 20, 65), (15, 1, 18, 64)])
+def test_convolution_reach_of_weights_without_numbers(K, d, H, W, value):
+    """An infinite or NaN weight makes its channel's outputs that value where its tap lies inside
+    the image, and NaN where the tap's pixel is padding: zero times it (x > 0, weights > 0)."""
+    N = 2
+    g = torch.Generator(device=DEV).manual_seed(K * H)
+    x = (torch.rand((N, H, W, C), generator=g, device=DEV) + 0.5).to(torch.bfloat16)
+    w = torch.rand((C, C, K, K), generator=g, device=DEV) + 0.5
+    w[3, 5, 0, 1] = value
+    w[31, 0, K - 1, K // 2] = value
+    want = torch.zeros(N, H, W, C, dtype=torch.int32)
+    for co, ky, kx in ((3, 0, 1), (31, K - 1, K // 2)):
+        y, xx = torch.meshgrid(torch.arange(H) + (ky - K // 2) * d,
+                               torch.arange(W) + (kx - K // 2) * d, indexing="ij")
+        inside = (y >= 0) & (y < H) & (xx >= 0) & (xx < W)
+        want[..., co] = torch.where(inside, 1 if value == value else 3, 3).int()
+    bias = torch.zeros(C, device=DEV)
+    assert torch.equal(_reach(_convolve(x, w, d, bias)), want)
