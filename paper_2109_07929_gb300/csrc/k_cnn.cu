@@ -317,6 +317,7 @@ struct TapPlan {
 // False where the old form is the better one (or the only one that fits).
 bool tap_plan(int K, int d, int W, TapPlan& p) {
   if (K < 5) return false;             // a row of 1 or 3 taps would leave M mostly zero
+  if (d > 256 / (kTapM - 1)) return false;             // (before the products below overflow)
   p.G = (K + kTapM - 1) / kTapM;
   long best = -1;
   for (int P = 16; P <= 240; P += 16) {
@@ -1293,8 +1294,11 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     count_launches(1);
     return launch_status("mca_cnn_conv launch");
   }
-  const ConvPlan plan = (cout_mma == 32) ? conv_plan<32>(ksize, dilation)
-                                         : conv_plan<16>(ksize, dilation);
+  // a row segment takes 64 bytes per pixel, 128 + (K - 1) d of them (compared in 64 bits: the
+  // plan's own arithmetic has 32)
+  const bool fits = (int64_t)(ksize - 1) * dilation <= 227 * 1024 / 64;
+  const ConvPlan plan = !fits ? ConvPlan{} : (cout_mma == 32) ? conv_plan<32>(ksize, dilation)
+                                                              : conv_plan<16>(ksize, dilation);
   if (plan.stages < 2 || plan.smem > 227 * 1024) {
     set_error_message("mca_cnn_conv: kernel size and dilation too large for one row segment");
     return MCA_ERR_INVALID_ARG;
@@ -1348,15 +1352,18 @@ int mca_cnn_conv_wgrad(const uint16_t* x, const uint16_t* gz, int32_t n, int32_t
     return MCA_ERR_UNSUPPORTED;
   }
   const int T = ksize * ksize;
+  // beyond the image's sizes every dilation is the same (only the centre tap sees pixels); the
+  // bound keeps the shifts within 32 bits
+  const int d = std::min(dilation, std::max(h, w));
   // partial sums: the scratch holds one set per kWgRows image rows
   const int nmax = (int)(((int64_t)n * h + kWgRows - 1) / kWgRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int nchunk;
   if (ksize >= 5 && ksize <= kWrMaxK) {
     WrArgs a{};
-    a.H = h; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
-    const int rem = h % (kWrJ * dilation);
-    a.blocks = h / (kWrJ * dilation) * dilation + (rem < dilation ? rem : dilation);
+    a.H = h; a.K = ksize; a.d = d; a.r = (ksize - 1) / 2;
+    const int64_t period = (int64_t)kWrJ * d;          // image rows of d row blocks
+    a.blocks = (int)(h / period * d + std::min<int64_t>(h % period, d));
     a.nxc = (w + kWgPix - 1) / kWgPix;
     a.items = n * a.blocks * a.nxc;
     a.part = scratch;
@@ -1379,7 +1386,7 @@ int mca_cnn_conv_wgrad(const uint16_t* x, const uint16_t* gz, int32_t n, int32_t
     k_wgrad_rows<<<dim3(ksize, nchunk), 128, smem, s>>>(tmX, tmG, a);
   } else {
     WgArgs a{};
-    a.N = n; a.H = h; a.W = w; a.K = ksize; a.d = dilation; a.r = (ksize - 1) / 2;
+    a.N = n; a.H = h; a.W = w; a.K = ksize; a.d = d; a.r = (ksize - 1) / 2;
     a.rows_total = n * h;
     a.nxc = (w + kWgPix - 1) / kWgPix;
     a.part = scratch;

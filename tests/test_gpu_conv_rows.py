@@ -147,3 +147,27 @@ def test_convolution_reach_of_weights_without_numbers(K, d, H, W, value):
         want[..., co] = torch.where(inside, 1 if value == value else 3, 3).int()
     bias = torch.zeros(C, device=DEV)
     assert torch.equal(_reach(_convolve(x, w, d, bias)), want)
+
+
+@pytest.mark.parametrize("K", [3, 5, 11, 13, 15])
+@pytest.mark.parametrize("d", [70, 2 ** 29, 2 ** 30, 2 ** 30 + 1, 2 ** 31 - 1])
+def test_dilations_beyond_the_image(K, d):
+    """The weight gradient of a dilation beyond the image is that of its centre tap, whatever the
+    dilation (four times it no longer fits 32 bits); the convolution refuses a row segment that
+    does not fit, whatever its 32-bit products wrap to."""
+    N, H, W = 2, 9, 70
+    g = torch.Generator(device=DEV).manual_seed(K)
+    x, gz = (torch.randn((N, H, W, C), generator=g, device=DEV).to(torch.bfloat16)
+             for _ in range(2))
+    gw, _, _ = _weight_gradient(x, gz, K, d)
+    centre = gz.double().reshape(-1, C).T @ x.double().reshape(-1, C)
+    size = gz.double().abs().reshape(-1, C).T @ x.double().abs().reshape(-1, C)
+    r = K // 2
+    assert bool(((gw[:, :, r, r].double() - centre).abs() <= 1e-5 * size).all())
+    gw[:, :, r, r] = 0
+    assert int(torch.count_nonzero(gw)) == 0
+    if d > 70:
+        out, wt = torch.empty_like(x), torch.zeros(K * K, C, C, device=DEV).to(torch.bfloat16)
+        for dd in (d, 1431655721, 1431655722, 1431655766):
+            assert mca.load().mca_cnn_conv(x.data_ptr(), N, H, W, wt.data_ptr(), K, dd, C, C, None, 0, 0,
+                                           None, out.data_ptr(), None, None) == mca.ERR_INVALID_ARG
