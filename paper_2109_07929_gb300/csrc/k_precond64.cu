@@ -52,7 +52,8 @@ constexpr int kOzStages = 2;
 constexpr int kOzBar = kOzStages * kOzStage;
 constexpr int kOzSmem = kOzBar + 256 + 1024;
 constexpr int kOzKMax = 512;      // largest K whose 8 products per weight FP32 sums hold exactly
-constexpr int kBadRow = 0x7FFFFFFF;   // exponent of a row with an infinity or a NaN
+constexpr int kBadRow = 0x7FFFFFFF;   // exponent of a row with an infinity or a NaN, which has
+                                      // no slices: its results are the plain FP64 sums
 constexpr int kZeroRow = -0x7FFFFFFF; // and of a row of zeros
 
 // Row slicing: a warp per row, `rows` of them (of the batch at hand; the operand holds
@@ -151,6 +152,9 @@ __device__ __forceinline__ double scale2(double x, int e) {
 struct OzArgs {
   int R, C, K0, K1;          // output rows per block, columns, this launch's K range
   const int *ea, *eb;        // exponents of A's rows (all blocks) and of Bm's
+  const double *A, *Bm;      // the operands themselves, K entries a row
+  BlkAddr a;
+  int K;
   double* O;
   BlkAddr o;
   const VecCtl* ctl;
@@ -247,6 +251,7 @@ k_gemm_sliced(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     const int r = r0 + q * 32 + lane;
     const bool rok = r < p.R;
     const int ea = rok ? p.ea[blk * p.R + r] : kZeroRow;
+    const double* A = p.A + (size_t)b * p.a.bs + (size_t)(blk & 1) * p.a.ls + (size_t)r * p.a.ld;
     double* O = p.O + (size_t)b * p.o.bs + (size_t)(blk & 1) * p.o.ls + r;
     const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
 #pragma unroll 1
@@ -259,6 +264,16 @@ k_gemm_sliced(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       for (int j = 0; j < 8; ++j) {
         const int c = c0 + half * 32 + cc * 8 + j;
         if (c >= p.C || !rok) continue;
+        double* dst = O + (size_t)c * p.o.ld;
+        if (ea == kBadRow) {                           // (in the first K range)
+          if (ADD) continue;
+          const double* q = p.Bm + (size_t)c * p.K;
+          double x = 0.0;
+#pragma unroll 1
+          for (int k = 0; k < p.K; ++k) x = fma(A[k], q[k], x);
+          *dst = x;
+          continue;
+        }
         const int eb = p.eb[c];
         int t[kSlices];
 #pragma unroll
@@ -266,11 +281,7 @@ k_gemm_sliced(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         // 2^(ea + eb + 4) sum_d t_d 128^-(d + 2)
         const double hi = join4(t[0], t[1], t[2], t[3]), lo = join4(t[4], t[5], t[6], t[7]);
         double x = fma(lo, 0x1p-28, hi);
-        if (ea == kBadRow || eb == kBadRow)
-          x = __longlong_as_double(0x7FF8000000000000LL);
-        else
-          x = (ea == kZeroRow || eb == kZeroRow) ? 0.0 : scale2(x, ea + eb + 4 - 5 * kDigit);
-        double* dst = O + (size_t)c * p.o.ld;
+        x = (ea == kZeroRow || eb == kZeroRow) ? 0.0 : scale2(x, ea + eb + 4 - 5 * kDigit);
         *dst = ADD ? *dst + x : x;
       }
     }
@@ -336,12 +347,14 @@ void launch_slice_rows(const double* A, BlkAddr a, int R, const SlicedOperand& o
                                               (size_t)op.rows * op.Kp, ctl, op.buf, op.exps);
 }
 
-int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, double* O, BlkAddr o,
-                       int B, int R, int C, const VecCtl* ctl, int* err, cudaStream_t s) {
+int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, const double* A64,
+                       BlkAddr a, const double* Bm64, double* O, BlkAddr o, int B, int R, int C,
+                       const VecCtl* ctl, int* err, cudaStream_t s) {
   const dim3 grid((R + kOzM - 1) / kOzM, (C + kOzN - 1) / kOzN, 2 * B);
   int launches = 0;
   for (int k0 = 0; k0 < A.Kp; k0 += kOzKMax, ++launches) {
-    const OzArgs p{R, C, k0, std::min(A.Kp, k0 + kOzKMax), A.exps, Bm.exps, O, o, ctl, err};
+    const OzArgs p{R, C, k0, std::min(A.Kp, k0 + kOzKMax), A.exps, Bm.exps, A64, Bm64, a,
+                   A.K, O, o, ctl, err};
     if (k0 == 0)
       k_gemm_sliced<false><<<grid, kOzThreads, kOzSmem, s>>>(A.map, Bm.map, p);
     else

@@ -654,27 +654,28 @@ int precond_apply(mca_handle* h, int precision, const double* rin, size_t rstrid
     const double f_r = 4.0 * m * (double)n * n, f_c = 4.0 * n * (double)m * m;
     // O[blk][c][r] = sum_k A[blk][r][k] Q[c][k] for the blocks of B vectors
     auto transform = [&](const double* A, BlkAddr a, const SlicedOperand& op,
-                         const SlicedOperand& q, double* O, BlkAddr o, int R, int K) {
+                         const SlicedOperand& q, const double* q64, double* O, BlkAddr o, int R,
+                         int K) {
       launch_slice_rows(A, a, R, op, 2 * B * R, ctl, s);
-      count_launches(1 + launch_gemm_sliced(op, q, O, o, B, R, K, ctl, h->err, s));
+      count_launches(1 + launch_gemm_sliced(op, q, A, a, q64, O, o, B, R, K, ctl, h->err, s));
     };
     BlkAddr a1{rstride, mn, (size_t)n}, o1{2 * mn, mn, (size_t)m};
     cudaEvent_t t0 = prof_begin(h, s);
-    transform(rin, a1, h->opA_mn, h->opQrT, h->T1_64, o1, m, n);
+    transform(rin, a1, h->opA_mn, h->opQrT, h->QrT, h->T1_64, o1, m, n);
     prof_end(h, t0, MCA_FAM_PRECOND_1, prof_k, 32.0 * mn, f_r, s);
     BlkAddr a2{2 * mn, mn, (size_t)m}, o2{2 * mn, mn, (size_t)n};
     t0 = prof_begin(h, s);
-    transform(h->T1_64, a2, h->opA_nm, h->opQcT, h->Xh_64, o2, n, m);
+    transform(h->T1_64, a2, h->opA_nm, h->opQcT, h->QcT, h->Xh_64, o2, n, m);
     launch_modes_2x2_f64(h->Xh_64, h->mu, h->nu, m, n, ctl, B, kidx, s);
     count_launches(1);
     prof_end(h, t0, MCA_FAM_PRECOND_2, prof_k, 64.0 * mn, f_c, s);
     BlkAddr a3{2 * mn, mn, (size_t)n}, o3{2 * mn, mn, (size_t)m};
     t0 = prof_begin(h, s);
-    transform(h->Xh_64, a3, h->opA_mn, h->opQr, h->E_64, o3, m, n);
+    transform(h->Xh_64, a3, h->opA_mn, h->opQr, h->Qr, h->E_64, o3, m, n);
     prof_end(h, t0, MCA_FAM_PRECOND_3, prof_k, 32.0 * mn, f_r, s);
     BlkAddr a4{2 * mn, mn, (size_t)m}, o4{zstride, mn, (size_t)n};
     t0 = prof_begin(h, s);
-    transform(h->E_64, a4, h->opA_nm, h->opQc, zout, o4, n, m);
+    transform(h->E_64, a4, h->opA_nm, h->opQc, h->Qc, zout, o4, n, m);
     prof_end(h, t0, MCA_FAM_PRECOND_4, prof_k, 32.0 * mn, f_c, s);
     MCA_CUDA_TRY(cudaGetLastError());
     return MCA_OK;

@@ -93,7 +93,10 @@ int make_sliced(SlicedOperand* op, __nv_bfloat16* buf, int* exps, int rows, int 
 // block) starts at A + b a.bs + layer a.ls + r a.ld; blocks of inactive vectors are skipped.
 void launch_slice_rows(const double* A, BlkAddr a, int R, const SlicedOperand& op, int rows,
                        const VecCtl* ctl, cudaStream_t s);
-// O[blk][c][r] = sum_k A[blk][r][k] Bm[c][k] for 2 B blocks; returns the launches made.
-int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, double* O, BlkAddr o,
-                       int B, int R, int C, const VecCtl* ctl, int* err, cudaStream_t s);
+// O[blk][c][r] = sum_k A[blk][r][k] Bm[c][k] for 2 B blocks; returns the launches made.  A64 (by
+// a, as in launch_slice_rows) and Bm64 are the operands in FP64, read for the rows of A with an
+// infinity or a NaN.
+int launch_gemm_sliced(const SlicedOperand& A, const SlicedOperand& Bm, const double* A64,
+                       BlkAddr a, const double* Bm64, double* O, BlkAddr o, int B, int R, int C,
+                       const VecCtl* ctl, int* err, cudaStream_t s);
 }  // namespace mca

@@ -1,0 +1,56 @@
+"""What the sliced FP64 transforms and the chunked line solves of the paper's M_hat owe to the
+plain FP64 forms they replaced: the same infinities and NaN, and their accuracy."""
+import numpy as np
+import pytest
+
+import mca_inputs as mi
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2109_07929_gb300 as mca  # noqa: E402
+
+DEV = "cuda:0"
+
+
+def _reach(t):
+    """0 finite, 1 infinity, 2 minus infinity, 3 NaN."""
+    return np.isposinf(t) * 1 + np.isneginf(t) * 2 + np.isnan(t) * 3
+
+
+def _chain(rows, q):
+    """out[c][r] = sum_k rows[r][k] q[c][k], one product after the other."""
+    out = np.zeros((q.shape[0], rows.shape[0]))
+    for k in range(q.shape[1]):
+        out = out + np.outer(q[:, k], rows[:, k])
+    return out
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 7), (7, 1), (5, 40), (33, 70), (2, 600)])
+def test_fp64_preconditioner_reach_of_infinities(m, n, value):
+    """An infinite or NaN entry of r gives the infinities and NaN of the plain FP64 sums (with the
+    handle's own eigenvectors); the other vector of the batch is not touched."""
+    cb = mi.make_crossbar(m, n, 4)
+    rng = np.random.default_rng(1)
+    a = np.array([2e-5, 0.2])
+    with mca.Solver(mca.default_params(m, n, precision=mca.PREC_FP64, max_batch=2),
+                    cb.gmap) as s:
+        mu, qr, nu, qc = s.eigenpairs()
+        for pos in (0, m * n - 1, m * n + m * n // 2):
+            r = rng.standard_normal((2, 2 * m * n))
+            rd = torch.as_tensor(r, device=DEV)
+            clean, z = torch.empty_like(rd), torch.empty_like(rd)
+            s.precond_apply(a, rd, clean)
+            rd[0, pos] = value
+            s.precond_apply(a, rd, z)
+            assert torch.equal(z[1], clean[1])
+            with np.errstate(invalid="ignore"):
+                h = [_chain(_chain(x.reshape(m, n), qr.T), qc.T)
+                     for x in rd[0].cpu().numpy().reshape(2, m * n)]
+                det = nu[:, None] * mu + a[0] * (nu[:, None] + mu)
+                t = ((nu[:, None] + a[0]) * h[0] + a[0] * h[1]) / det
+                b = (a[0] * h[0] + (mu + a[0]) * h[1]) / det
+                ref = [_chain(_chain(y, qr), qc) for y in (t, b)]
+            assert np.array_equal(_reach(z[0].cpu().numpy()),
+                                  _reach(np.concatenate([x.ravel() for x in ref])))
