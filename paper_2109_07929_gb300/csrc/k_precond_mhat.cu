@@ -166,18 +166,23 @@ k_mhat_factor(int m, int n, Grid gr, const VecCtl* __restrict__ ctl, double* __r
 }
 
 // Value that enters chunk `lane` from its left (right): inclusive scan of the chunks' own end
-// values v with the factors f (5 x 32), then shifted by one.
+// values v with the factors f (5 x 32), then shifted by one.  Lanes without a partner keep v
+// (their factor is zero, which an infinite v would turn into NaN).
 __device__ __forceinline__ double carry_left(double v, const double* __restrict__ f, int lane) {
 #pragma unroll
-  for (int s = 0; s < 5; ++s)
-    v = fma(f[s * kChunks + lane], __shfl_up_sync(0xffffffffu, v, 1 << s), v);
+  for (int s = 0; s < 5; ++s) {
+    const double w = fma(f[s * kChunks + lane], __shfl_up_sync(0xffffffffu, v, 1 << s), v);
+    v = (lane >= (1 << s)) ? w : v;
+  }
   v = __shfl_up_sync(0xffffffffu, v, 1);
   return lane == 0 ? 0.0 : v;
 }
 __device__ __forceinline__ double carry_right(double v, const double* __restrict__ f, int lane) {
 #pragma unroll
-  for (int s = 0; s < 5; ++s)
-    v = fma(f[s * kChunks + lane], __shfl_down_sync(0xffffffffu, v, 1 << s), v);
+  for (int s = 0; s < 5; ++s) {
+    const double w = fma(f[s * kChunks + lane], __shfl_down_sync(0xffffffffu, v, 1 << s), v);
+    v = (lane + (1 << s) < kChunks) ? w : v;
+  }
   v = __shfl_down_sync(0xffffffffu, v, 1);
   return lane == kChunks - 1 ? 0.0 : v;
 }

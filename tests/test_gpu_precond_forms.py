@@ -54,3 +54,29 @@ def test_fp64_preconditioner_reach_of_infinities(m, n, value):
                 ref = [_chain(_chain(y, qr), qc) for y in (t, b)]
             assert np.array_equal(_reach(z[0].cpu().numpy()),
                                   _reach(np.concatenate([x.ravel() for x in ref])))
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 7), (7, 1), (5, 40), (33, 70), (300, 33)])
+def test_mhat_reach_of_infinities(m, n, value):
+    """z_b = G_2^-1 r_b along columns and z_t = (r_t + a z_b) G_1^-1 along rows, with inverses
+    whose entries are all positive: an entry of r_t reaches its row of z_t as it is, one of r_b
+    its column of z_b and with it every entry of z_t."""
+    cb = mi.make_crossbar(m, n, 4)
+    kind = 3 if value != value else (1 if value > 0 else 2)
+    r = np.random.default_rng(1).standard_normal((1, 2, m, n))
+    with mca.Solver(mca.default_params(m, n, precision=mca.PREC_MHAT, max_batch=1),
+                    cb.gmap) as s:
+        for layer in (0, 1):
+            for i, j in {(0, 0), (m // 2, n // 2), (m - 1, n - 1)}:
+                rd = torch.as_tensor(r, device=DEV)
+                rd[0, layer, i, j] = value
+                z = torch.empty_like(rd)
+                s.precond_apply(np.array([2e-4]), rd.view(1, -1), z.view(1, -1))
+                want = np.zeros((2, m, n), int)
+                if layer == 0:
+                    want[0, i] = kind
+                else:
+                    want[0] = kind
+                    want[1, :, j] = kind
+                assert np.array_equal(_reach(z[0].cpu().numpy()), want)
