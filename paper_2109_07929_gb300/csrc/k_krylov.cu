@@ -16,6 +16,8 @@
 // is skipped; the GMRES residual estimate is then exact up to a factor 1 + O(k kOrthTol).
 // All reductions are two-level (per-block partials, then one fixed-order sum per vector),
 // hence deterministic.
+#include <algorithm>
+
 #include "bits.cuh"
 #include "mca_internal.cuh"
 #include "solver_dev.cuh"
@@ -78,8 +80,11 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
 // not depend on how many accumulators a thread holds.
 
 // pass 3 (marked vectors only): partial dots <V_j, u> of the new vector u, reduced by the
-// last block into h2_j = s_j <V_j, u>.  Rarely does any work, so a launch has a quarter of
-// the summation's blocks, each taking them in turn.
+// last block into h2_j = s_j <V_j, u>.  Most launches find no marked vector and only end their
+// blocks, so a launch has a quarter of the summation's blocks, each taking them in turn, where
+// that leaves the eight per SM that reside, and for few vectors as many as do: with a quarter
+// of the blocks the pass and its update took 352 us for one vector of 1024 x 1024 (long cycles,
+// Jacobi preconditioner; now 233) and 50 us at 64 x 64 (now 34).
 // ZS: the Newton step from V = 0, whose v_0 is stored in the first column of the top layer
 // only (the residual's sparse_f); its other entries are not read, and the last block also
 // subtracts h2_0 v_0 from u (see subtract_sparse_v0), in place of the update pass.
@@ -463,7 +468,9 @@ void launch_reduce_dots(const double* part, int nblk, int nk, double* h, int B,
 void launch_reorth_dots(double* u, const double* V, size_t vstride, size_t n2, int nk,
                         double* part, int nblk, int B, const VecCtl* ctl, unsigned int* cnt,
                         double* h2, cudaStream_t s, bool zs, int ncols) {
-  const dim3 grid((nblk + 3) / 4, B);
+  constexpr int kResident = 8 * 152;
+  const int turns = std::max(1, std::min(4, nblk * B / kResident));
+  const dim3 grid((nblk + turns - 1) / turns, B);
 #define MCA_CALL(KP_)                                                                        \
   do {                                                                                       \
     if (zs)                                                                                  \
