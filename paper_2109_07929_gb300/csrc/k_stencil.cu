@@ -969,72 +969,99 @@ void launch_init_basis(const double* F, double sign, double* V0, size_t vstride,
   k_init_basis<<<dim3(nb, B), kThreads, 0, s>>>(F, sign, V0, vstride, xbf, mp, np, m, n, ctl);
 }
 
-template <typename ZT, int AM, bool ZS = false>
+// Pairs of cells: every row starts on a pair, and every array on a 16-byte boundary.
+template <typename ZT>
+bool in_pairs(const Grid& gr, const double* D, const ZT* z, size_t zstride, const double* w,
+              const double* V, size_t vstride) {
+  auto on = [](const void* p, size_t a) {
+    return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0;
+  };
+  return (gr.n & 1) == 0 && on(D, 16) && on(w, 16) && on(V, 16) && on(z, 2 * sizeof(ZT)) &&
+         (zstride & 1) == 0 && (vstride & 1) == 0;
+}
+
+// z: the vector of batch entry 0, later entries zstride apart
+template <typename ZT, int AM>
+void apply_only(const Grid& gr, const double* D, const ZT* z, size_t zstride, double* w, int nblk,
+                int B, cudaStream_t s) {
+  const FastDiv by_n(gr.n);
+  if (in_pairs(gr, D, z, zstride, w, nullptr, 0))
+    k_spmv_dots<1, ZT, AM, false, 2><<<dim3((nblk + 1) / 2, B), kThreads, 0, s>>>(
+        gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
+  else
+    k_spmv_dots<1, ZT, AM, false, 1><<<dim3(nblk, B), kThreads, 0, s>>>(
+        gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
+}
+
+// V: basis vector 0 of batch entry 0 (nk vectors N2 apart, entries vstride apart)
+template <typename ZT, int AM, bool ZS>
 void spmv_dots(const Grid& gr, const double* D, const ZT* z, size_t zstride, double* w,
                const double* V, size_t vstride, int nk, double* part, int nblk, int B,
                const VecCtl* ctl, unsigned int* cnt, double* h, cudaStream_t s) {
-  // z: the vector of batch entry 0, later entries zstride doubles apart; V: basis vector
-  // 0 of batch entry 0 (nk vectors N2 apart, entries vstride apart), or NULL.
-  // pairs of cells: every row starts on a pair, and every array on a 16-byte boundary
-  auto on = [](const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
-  const bool two = (gr.n & 1) == 0 && on(D, 16) && on(w, 16) && on(V, 16) &&
-                   on(z, 2 * sizeof(ZT)) && (zstride & 1) == 0 && (vstride & 1) == 0;
+  const bool two = in_pairs(gr, D, z, zstride, w, V, vstride);
   const FastDiv by_n(gr.n);
-  // the arithmetics the solver runs with dots; the others only serve mca_jacobian_apply_f32
-  constexpr bool kDots = std::is_same<ZT, double>::value || AM == kApplyPair || ZS;
 #define MCA_SPMV1(KP_, W_)                                                                   \
   k_spmv_dots<KP_, ZT, AM, ZS, W_><<<dim3((nblk + W_ - 1) / W_, B), kThreads, 0, s>>>(       \
       gr, D, z, zstride, w, V, vstride, nk, part, nblk, ctl, cnt, h, by_n)
 #define MCA_SPMV(KP_) do { if (two) MCA_SPMV1(KP_, 2); else MCA_SPMV1(KP_, 1); } while (0)
-  if (V == nullptr) {
-    MCA_SPMV(1);
-  } else if constexpr (kDots) {
-    switch (nk) {
-      case 0: case 1: MCA_SPMV(1); break;
-      case 2: MCA_SPMV(2); break;
-      case 3: MCA_SPMV(3); break;
-      case 4: MCA_SPMV(4); break;
-      case 5: MCA_SPMV(5); break;
-      case 6: MCA_SPMV(6); break;
-      case 7: MCA_SPMV(7); break;
-      case 8: MCA_SPMV(8); break;
-      default:
-        if (nk <= 10) MCA_SPMV1(10, 1);
-        else if (nk <= 12) MCA_SPMV1(12, 1);
-        else if (nk <= 16) MCA_SPMV1(16, 1);
-        else if (nk <= 20) MCA_SPMV1(20, 1);
-        else if (nk <= 24) MCA_SPMV1(24, 1);
-        else MCA_SPMV1(32, 1);
-    }
+  switch (nk) {
+    case 0: case 1: MCA_SPMV(1); break;
+    case 2: MCA_SPMV(2); break;
+    case 3: MCA_SPMV(3); break;
+    case 4: MCA_SPMV(4); break;
+    case 5: MCA_SPMV(5); break;
+    case 6: MCA_SPMV(6); break;
+    case 7: MCA_SPMV(7); break;
+    case 8: MCA_SPMV(8); break;
+    default:
+      if (nk <= 10) MCA_SPMV1(10, 1);
+      else if (nk <= 12) MCA_SPMV1(12, 1);
+      else if (nk <= 16) MCA_SPMV1(16, 1);
+      else if (nk <= 20) MCA_SPMV1(20, 1);
+      else if (nk <= 24) MCA_SPMV1(24, 1);
+      else MCA_SPMV1(32, 1);
   }
 #undef MCA_SPMV
 #undef MCA_SPMV1
+}
+
+void launch_apply(const Grid& gr, const double* D, const double* z, double* w, int nblk, int B,
+                  cudaStream_t s) {
+  apply_only<double, kApplyF64>(gr, D, z, 2 * (size_t)gr.m * gr.n, w, nblk, B, s);
+}
+
+void launch_apply(const Grid& gr, const double* D, const float* z, double* w, int nblk, int B,
+                  ApplyMode mode, cudaStream_t s) {
+  const size_t n2 = 2 * (size_t)gr.m * gr.n;
+  switch (mode) {
+    case kApplyF64: apply_only<float, kApplyF64>(gr, D, z, n2, w, nblk, B, s); break;
+    case kApplyF32: apply_only<float, kApplyF32>(gr, D, z, n2, w, nblk, B, s); break;
+    case kApplyPair: apply_only<float, kApplyPair>(gr, D, z, n2, w, nblk, B, s); break;
+  }
 }
 
 void launch_spmv_dots(const Grid& gr, const double* D, const double* z, size_t zstride,
                       double* w, const double* V, size_t vstride, int nk, double* part,
                       int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
                       cudaStream_t s) {
-  spmv_dots<double, kApplyF64>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl, cnt, h,
-                           s);
+  spmv_dots<double, kApplyF64, false>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl,
+                                      cnt, h, s);
 }
 
 void launch_spmv_dots(const Grid& gr, const double* D, const float* z, size_t zstride,
                       double* w, const double* V, size_t vstride, int nk, double* part,
                       int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
-                      cudaStream_t s, int apply) {
-  if (apply == kApplyF32Zero)
-    spmv_dots<float, kApplyF32, true>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl,
-                                      cnt, h, s);
-  else if (apply == kApplyF32)
-    spmv_dots<float, kApplyF32>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl, cnt,
-                                h, s);
-  else if (apply == kApplyF64)
-    spmv_dots<float, kApplyF64>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl, cnt,
-                                h, s);
-  else
-    spmv_dots<float, kApplyPair>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl, cnt,
-                                 h, s);
+                      cudaStream_t s) {
+  spmv_dots<float, kApplyPair, false>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl,
+                                    cnt, h, s);
+}
+
+void launch_spmv_dots_zero(const Grid& gr, const double* D, const float* z, size_t zstride,
+                           double* w, const double* V, size_t vstride, int nk, double* part,
+                           int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
+                           cudaStream_t s) {
+  spmv_dots<float, kApplyF32, true>(gr, D, z, zstride, w, V, vstride, nk, part, nblk, B, ctl,
+                                         cnt, h, s);
 }
 
 void launch_outputs(const Grid& gr, const double* vin, const double* x, double* i_out,

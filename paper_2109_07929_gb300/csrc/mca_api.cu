@@ -727,8 +727,12 @@ int enqueue_iteration(mca_handle* h, const double* D, int B, int k, cudaStream_t
     t0 = prof_begin(h, s);
     // the FP32 apply runs in the Newton step from V = 0, whose v_0 the residual stored in
     // the first column of the top layer only (sparse_f): its dots read v_0 there only
-    launch_spmv_dots(h->gr, D, zk, zstride, h->W, h->V, vstride, k + 1, h->part, nbS, B,
-                     h->ctl, h->cnt, h->h1, s, f32 ? kApplyF32Zero : kApplyPair);
+    if (f32)
+      launch_spmv_dots_zero(h->gr, D, zk, zstride, h->W, h->V, vstride, k + 1, h->part, nbS, B,
+                            h->ctl, h->cnt, h->h1, s);
+    else
+      launch_spmv_dots(h->gr, D, zk, zstride, h->W, h->V, vstride, k + 1, h->part, nbS, B, h->ctl,
+                       h->cnt, h->h1, s);
   } else {
     double* zk = h->Z + (size_t)k * n2;
     MCA_TRY(precond_apply(h, h->p.precision, vk, vstride, zk, zstride, B, h->ctl, s, k, D, k));
@@ -1704,8 +1708,7 @@ int mca_jacobian_apply(mca_handle* h, const double* D, const double* z, double* 
     return MCA_ERR_INVALID_ARG;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  launch_spmv_dots(h->gr, D, z, h->n2, w, nullptr, 0, 0, h->part, residual_nblk((int)h->mn),
-                   nvec, nullptr, nullptr, nullptr, s);
+  launch_apply(h->gr, D, z, w, residual_nblk((int)h->mn), nvec, s);
   count_launches(1);
   MCA_CUDA_TRY(cudaGetLastError());
   MCA_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1719,7 +1722,7 @@ int mca_jacobian_apply_f32(mca_handle* h, const double* D, const float* z, doubl
     set_error("bad arguments (nvec must be in 1..max_batch)");
     return MCA_ERR_INVALID_ARG;
   }
-  int apply;
+  ApplyMode apply;
   switch (mode) {
     case MCA_APPLY_PAIR: apply = kApplyPair; break;
     case MCA_APPLY_F64: apply = kApplyF64; break;
@@ -1729,8 +1732,7 @@ int mca_jacobian_apply_f32(mca_handle* h, const double* D, const float* z, doubl
       return MCA_ERR_INVALID_ARG;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  launch_spmv_dots(h->gr, D, z, h->n2, w, nullptr, 0, 0, h->part, residual_nblk((int)h->mn),
-                   nvec, nullptr, nullptr, nullptr, s, apply);
+  launch_apply(h->gr, D, z, w, residual_nblk((int)h->mn), nvec, apply, s);
   count_launches(1);
   MCA_CUDA_TRY(cudaGetLastError());
   MCA_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1844,8 +1846,7 @@ int mca_gmres_solve(mca_handle* h, const double* D, const double* a, const doubl
     if (!more || max_iters <= 0) break;
     // restart from the true residual r = rhs - J dx (vectors already converged restart
     // with a residual below their tolerance and do no further work)
-    launch_spmv_dots(h->gr, D, dx, n2, h->W, nullptr, 0, 0, h->part, nbS, nvec, nullptr,
-                     nullptr, nullptr, s);
+    launch_apply(h->gr, D, dx, h->W, nbS, nvec, s);
     launch_sub(rhs, h->W, h->F, n2, nvec, s);
     count_launches(2);
   }

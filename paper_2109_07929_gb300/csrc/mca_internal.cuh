@@ -211,7 +211,7 @@ double pair_err_bound(double size2_sum);
 // residual for exactly those vectors.
 // sparse_f (zero_state only): F = -Y is stored in the first column of the top layer only
 // (its other entries are zero and left unwritten); the step's kernels must then read v_0
-// there only (kApplyF32Zero, the update passes' zs).
+// there only (launch_spmv_dots_zero, the update passes' zs).
 void launch_residual_newton(const Grid& gr, const double* gmaps, const int* map_of,
                             const double* vin, const double* x, bool zero_state, double* F,
                             size_t fstride, __nv_bfloat16* xbf, int mp, int np, double* D,
@@ -221,14 +221,7 @@ void launch_residual_newton(const Grid& gr, const double* gmaps, const int* map_
 void launch_init_basis(const double* F, double sign, double* V0, size_t vstride,
                        __nv_bfloat16* xbf, int mp, int np, int m, int n, const VecCtl* ctl,
                        int B, cudaStream_t s);
-// w = J z fused with the partial dots <V_j, w> (j < nk); with cnt != NULL the last block
-// of each vector also reduces them into h[b][j].
-void launch_spmv_dots(const Grid& gr, const double* D, const double* z, size_t zstride,
-                      double* w, const double* V, size_t vstride, int nk, double* part,
-                      int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
-                      cudaStream_t s);
-// The same with z in FP32 (the tensor-core preconditioner's output).  apply picks the
-// arithmetic of w = J z; the dots stay FP64 in every mode:
+// Arithmetic of w = J z with z in FP32 (the tensor-core preconditioner's output):
 //   kApplyPair: FP32 pairs (error-free products and sums of the FP32 z with the wire
 //     constants and D split into FP32 pairs), rounded once to FP64; the error stays
 //     within about 2^-45 of the size of the terms, against 2^-51 for kApplyF64, and the FP64
@@ -236,13 +229,29 @@ void launch_spmv_dots(const Grid& gr, const double* D, const double* z, size_t z
 //   kApplyF64: FP64 on z widened exactly;
 //   kApplyF32: plain FP32 (w rounded to FP32, then widened), for linear solves whose
 //     forcing term is loose (kF32ApplyMinEta).
-//   kApplyF32Zero: kApplyF32 in the Newton step from V = 0 whose v_0 is stored in the first
-//     column of the top layer only (the residual's sparse_f): the dots read it there only.
-enum ApplyMode { kApplyF64 = 0, kApplyF32 = 1, kApplyPair = 2, kApplyF32Zero = 3 };
+enum ApplyMode { kApplyF64 = 0, kApplyF32 = 1, kApplyPair = 2 };
+// w = J z of B vectors, one after the other in z and w
+void launch_apply(const Grid& gr, const double* D, const double* z, double* w, int nblk, int B,
+                  cudaStream_t s);
+void launch_apply(const Grid& gr, const double* D, const float* z, double* w, int nblk, int B,
+                  ApplyMode mode, cudaStream_t s);
+// w = J z fused with the partial dots <V_j, w> (j < nk, V and ctl not NULL); with cnt != NULL
+// the last block of each vector also reduces them into h[b][j].
+void launch_spmv_dots(const Grid& gr, const double* D, const double* z, size_t zstride,
+                      double* w, const double* V, size_t vstride, int nk, double* part,
+                      int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
+                      cudaStream_t s);
+// The same with z in FP32, by kApplyPair (the dots stay FP64).
 void launch_spmv_dots(const Grid& gr, const double* D, const float* z, size_t zstride,
                       double* w, const double* V, size_t vstride, int nk, double* part,
                       int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
-                      cudaStream_t s, int apply);
+                      cudaStream_t s);
+// The same by kApplyF32 in the Newton step from V = 0, whose v_0 is stored in the first column of
+// the top layer only (the residual's sparse_f): the dots read it there only.
+void launch_spmv_dots_zero(const Grid& gr, const double* D, const float* z, size_t zstride,
+                           double* w, const double* V, size_t vstride, int nk, double* part,
+                           int nblk, int B, const VecCtl* ctl, unsigned int* cnt, double* h,
+                           cudaStream_t s);
 // Smallest forcing term at which a Newton step's Jacobian applies run in FP32.  FP32
 // rounding of J z is relative to the wire terms, which cancel heavily, so it leaves a
 // floor on the linear residual (near 1e-5 relative in an FP32 model of the solver); the
