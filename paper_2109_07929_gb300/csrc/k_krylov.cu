@@ -57,7 +57,7 @@ __device__ __forceinline__ bool last_block(unsigned int* cnt, int b) {
   return last;
 }
 
-// h[b][j] = sum over blocks of part[b][j][:] for j < nk.
+// h[b][j] = sum over blocks of part[b][j][:] for j < nk (kHStride; nothing behind them).
 __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
                               double* __restrict__ h, const VecCtl* __restrict__ ctl) {
   const int b = blockIdx.x;
@@ -67,7 +67,7 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
     double s = 0.0;
     for (int t = l; t < nblk; t += 32) s += part[((size_t)b * 32 + j) * nblk + t];
     s = warp_sum(s);
-    if (l == 0) h[(size_t)b * 32 + j] = s;
+    if (l == 0) h[(size_t)b * kHStride + j] = s;
   }
 }
 

@@ -1658,13 +1658,13 @@ int mca_residual(mca_handle* h, const double* x, const double* v_in, int32_t nve
   launch_reduce_dots(h->part, nb, 2, h->h1, nvec, nullptr, s);
   count_launches(1);
   MCA_CUDA_TRY(cudaGetLastError());
-  std::vector<double> hh((size_t)nvec * 32);
+  std::vector<double> hh((size_t)nvec * kHStride);
   MCA_CUDA_TRY(cudaMemcpyAsync(hh.data(), h->h1, hh.size() * sizeof(double),
                                cudaMemcpyDeviceToHost, s));
   MCA_CUDA_TRY(cudaStreamSynchronize(s));
   for (int b = 0; b < nvec; ++b) {
-    if (fnorm) fnorm[b] = std::sqrt(hh[(size_t)b * 32]);
-    if (dmean) dmean[b] = hh[(size_t)b * 32 + 1] / (double)h->mn;
+    if (fnorm) fnorm[b] = std::sqrt(hh[(size_t)b * kHStride]);
+    if (dmean) dmean[b] = hh[(size_t)b * kHStride + 1] / (double)h->mn;
   }
   return MCA_OK;
 }
@@ -1688,14 +1688,14 @@ int mca_residual_pair(mca_handle* h, const double* x, const double* v_in, int32_
   launch_reduce_dots(h->part, nb, 3, h->h1, nvec, nullptr, s);
   count_launches(1);
   MCA_CUDA_TRY(cudaGetLastError());
-  std::vector<double> hh((size_t)nvec * 32);
+  std::vector<double> hh((size_t)nvec * kHStride);
   MCA_CUDA_TRY(cudaMemcpyAsync(hh.data(), h->h1, hh.size() * sizeof(double),
                                cudaMemcpyDeviceToHost, s));
   MCA_CUDA_TRY(cudaStreamSynchronize(s));
   for (int b = 0; b < nvec; ++b) {
-    if (fnorm) fnorm[b] = std::sqrt(hh[(size_t)b * 32]);
-    if (dmean) dmean[b] = hh[(size_t)b * 32 + 1] / (double)h->mn;
-    if (ferr) ferr[b] = pair_err_bound(hh[(size_t)b * 32 + 2]);
+    if (fnorm) fnorm[b] = std::sqrt(hh[(size_t)b * kHStride]);
+    if (dmean) dmean[b] = hh[(size_t)b * kHStride + 1] / (double)h->mn;
+    if (ferr) ferr[b] = pair_err_bound(hh[(size_t)b * kHStride + 2]);
   }
   return MCA_OK;
 }
