@@ -52,8 +52,13 @@ extern "C" {
 #define MCA_ERR_UNSUPPORTED (-7)   /* precision mode not available on this device       */
 
 /* ---- precision of the preconditioner apply (Section 3.2) -------------------------- */
-#define MCA_PREC_FP64 0        /* all four eigenbasis transforms with FP64 results (BF16
-                                  slices on the tensor cores, summed exactly)            */
+#define MCA_PREC_FP64 0        /* all four eigenbasis transforms with FP64 results, from rows
+                                  held as 55-bit fixed point on the tensor cores: at most
+                                  2^-50.8 of the two row maxima's product is left out per
+                                  product of entries, and the rest is summed exactly and
+                                  rounded once per 512 of K.  The error in the norm is below
+                                  that of FP64 sums; an entry far below its row's maximum
+                                  counts with fewer bits than its own 53                 */
 #define MCA_PREC_BF16 1        /* all four transforms on tcgen05 tensor cores, BF16 in,
                                   FP32 accumulate                                        */
 #define MCA_PREC_BF16_SPLIT 2  /* forward transforms BF16; back transforms with the

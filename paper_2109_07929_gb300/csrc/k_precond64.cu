@@ -9,20 +9,26 @@
 // holds it with FP64 results; the mixed-precision form lives in k_precond_tc.cu.
 //
 // The FP64 pipe gives 1.05 TFLOP/s, so the GEMM runs on the BF16 tensor cores, after Ozaki,
-// Ogita, Oishi and Rump
-// ("Error-free transformations of matrix multiplication by using fast routines of matrix
-// multiplication and its applications", Numer. Algorithms 59, 2012) and its tensor-core form
-// by Mukunoki, Ozaki, Ogita and Imamura (ISC 2020): every row of A and of Bm is scaled by a
-// power of two and cut into 8 slices of signed 7-bit digits,
-//   x = 2^(e + 2) sum_s a_s 128^-(s + 1),   |a_s| <= 64,
+// Ogita, Oishi and Rump ("Error-free transformations of matrix multiplication by using fast
+// routines of matrix multiplication and its applications", Numer. Algorithms 59, 2012) and its
+// tensor-core form by Mukunoki, Ozaki, Ogita and Imamura (ISC 2020): every row of A and of Bm is
+// scaled by a power of two and cut into 8 slices of signed 7-bit digits,
+//   x = 2^(e + 2) sum_s a_s 128^-(s + 1),   |a_s| <= 64,   2^e <= row maximum < 2^(e + 1),
 // which BF16 holds exactly; products of digits are integers of at most 2^12, so that the FP32
 // accumulators of the tensor core hold exactly what the up to 8 slice products of one weight
-// d = s + t sum over K <= 512 (8 x 512 x 2^12 = 2^24); and the sums of weights 0 .. 7 (36 of
-// the 64 slice products) are joined to one FP64 result per 512 of K, rounded once.  What is
-// dropped lies below 2^-54 of (row maximum) x (column maximum) per product, where a chain of
-// FMAs rounds at 2^-53 of its partial sums at every
-// step: the apply's error against quadruple precision is half that of the FMA chain's
-// (256 x 256: 5.8e-16 against 1.2e-15).
+// d = s + t sum over K <= 512 (8 x 512 x 2^12 = 2^24); and the sums of weights 0 .. 7 (36 of the
+// 64 slice products) are joined to one FP64 result per 512 of K, rounded once.
+//
+// What is lost, per product of entries and in units of 2^(ea + eb): the 28 products of weights 8
+// and up, at most 7.1 x 2^-54 (seven of weight 8 with 2^-54 each), and the rounding of the two
+// entries to multiples of 2^(e - 54), at most 2 x 2^-54: below 9.1 x 2^-54 = 2^-50.8, and 1.1 x
+// 2^-54 in the mean square over evenly spread digits.  So the error is relative to the maxima of
+// the rows, not to the entries: one 2^-20 of its row's maximum keeps 35 bits, one below 2^-56
+// none, where a chain of FMAs keeps 53 of each and rounds at 2^-53 of its partial sums.  The
+// apply's error in the norm falls all the same (96 x 160 to 40 x 600, random, spike, one-column,
+// graded, decaying and smooth right-hand sides, a from 2e-5 to 5: 2.7e-16 to 8.2e-16 of |z|, the
+// chain's 7.2e-16 to 2.1e-15); single small components move both ways, a spike's far field and
+// the largest of a smooth z's by up to 6 times the chain's error, others below it.
 // One apply (four transforms), against the FMA kernel: 512 x 512, 4 vectors 520 us (8300),
 // 1024 x 1024 933 us (16500), 64 x 64 135 us (324), 16 x 16 110 us (126).
 #include <cuda.h>
@@ -57,9 +63,10 @@ constexpr int kBadRow = 0x7FFFFFFF;   // exponent of a row with an infinity or a
 constexpr int kZeroRow = -0x7FFFFFFF; // and of a row of zeros
 
 // Row slicing: a warp per row, `rows` of them (of the batch at hand; the operand holds
-// plane / Kp).  out[s][row][k] (BF16, K padded to Kp with zeros) and exps[row].  Row r of
-// block blk = 2 b + layer starts at A + b a.bs + layer a.ls + r a.ld.  Integer arithmetic only: the entry's mantissa shifted to a 56-bit fixed-point
-// number in units of 2^(e - 54), its digits taken from the low end with a carry.
+// plane / Kp).  out[s][row][k] (BF16, K padded to Kp with zeros) and exps[row].  Row r of block
+// blk = 2 b + layer starts at A + b a.bs + layer a.ls + r a.ld.  Integer arithmetic only: the
+// entry's mantissa shifted to a 56-bit fixed-point number in units of 2^(e - 54), its digits
+// taken from the low end with a carry.
 __global__ void __launch_bounds__(256)
 k_slice_rows(const double* __restrict__ A, BlkAddr a, int R, int K, int Kp, int rows,
              size_t plane, const VecCtl* __restrict__ ctl, __nv_bfloat16* __restrict__ out,
