@@ -101,3 +101,64 @@ def test_fp64_preconditioner_loses_no_weight(m, n):
         ref = S.exact(r[v], qr, qc, mu, nu, a[v])
         err = float(np.sqrt(((z[v] - ref) ** 2).sum()))
         assert err <= 3 * S.expected_error(r[v], qr, qc, mu, nu, a[v])
+
+
+def _line(n, g, first, last, a):
+    """Diagonal of tridiag(-g, d + a, -g) over a line of n nodes between two terminations."""
+    d = np.full(n, 2.0 * g)
+    if n == 1:
+        d[0] = first + last
+    else:
+        d[0], d[-1] = first + g, g + last
+    return d + a
+
+
+def _times(d, g, x, sign=-1.0):
+    """The line operator along axis 0, in extended precision; sign = 1: its absolute values."""
+    x = x.astype(np.longdouble)
+    y = d.astype(np.longdouble)[:, None] * x
+    y[1:] += sign * g * x[:-1]
+    y[:-1] += sign * g * x[1:]
+    return y
+
+
+def _solve_line(d, g, w):
+    """Thomas sweeps along axis 0 (all terms of one sign for w >= 0)."""
+    piv, y = d.copy(), w.copy()
+    for j in range(1, len(d)):
+        q = g / piv[j - 1]
+        piv[j] -= q * g
+        y[j] += q * y[j - 1]
+    y[-1] /= piv[-1]
+    for j in range(len(d) - 2, -1, -1):
+        y[j] = (y[j] + g * y[j + 1]) / piv[j]
+    return y
+
+
+@pytest.mark.parametrize("m,n", [(2, 2), (1, 31), (32, 33), (65, 2), (100, 1025), (2049, 3),
+                                 (1057, 40)])
+def test_mhat_solves_are_backward_stable(m, n):
+    """G_2 z_b = r_b and z_t G_1 = r_t + a z_b to rounding, for a / g on both sides of the closed
+    form's two branches and at both ends.  A chunk of L nodes forms its carries' factors as
+    products of up to L terms, in both sweeps, so the residual is within (8 + 2 L) 2^-53 of
+    |G| |z|, with |z| the solution for |r| (an M-matrix: all its terms are positive)."""
+    cb = mi.make_crossbar(m, n, 4, g_wire_bot=0.5)
+    p = cb.params
+    a = np.array([1e-9, 2.1e-5, 0.2, 3.0, 1e6])
+    r = np.random.default_rng(7).standard_normal((len(a), 2, m, n))
+    prm = mca.default_params(m, n, g_wire_bot=0.5, precision=mca.PREC_MHAT, max_batch=len(a))
+    with mca.Solver(prm, cb.gmap) as s:
+        rd = torch.as_tensor(r.reshape(len(a), -1), device=DEV)
+        z = torch.empty_like(rd)
+        s.precond_apply(a, rd, z)
+    z = z.cpu().numpy().reshape(r.shape)
+    for v, av in enumerate(a):
+        for g, first, last, x, rhs, extra in (
+                (p.g_wire_bot, p.g_term_bot_top, p.g_sense, z[v, 1], r[v, 1], 0.0),
+                (p.g_wire_top, p.g_src, p.g_term_top_right, z[v, 0].T, r[v, 0].T, z[v, 1].T)):
+            d = _line(x.shape[0], g, first, last, av)
+            w = rhs + np.longdouble(av) * extra
+            size = np.abs(rhs) + av * np.abs(extra)
+            bound = (8 + 2 * -(-x.shape[0] // 32)) * 2.0 ** -53 * _times(
+                d, g, _solve_line(d, g, size), 1.0)
+            assert bool((np.abs(_times(d, g, x) - w) <= bound).all()), (av, g)
