@@ -71,12 +71,11 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
   }
 }
 
-// The reductions below follow one summation order, whatever the launch shape: nblk blocks
-// of kThreads accumulators per vector (vec_nblk; the Jacobian
-// apply: residual_nblk), accumulator (v, t) adding the
-// entries v kThreads + t + k nblk kThreads in order; then a butterfly over each 32
-// accumulators, the warps of a block in order, and the blocks' partial sums by 32 lanes and
-// a butterfly.  Results (and with them the rounding of the BF16 preconditioner's inputs) do
+// The reductions below follow one summation order, whatever the launch shape: nblk blocks of
+// kThreads accumulators per vector (vec_nblk; the Jacobian apply: residual_nblk), accumulator
+// (v, t) adding the entries v kThreads + t + k nblk kThreads in order; then a butterfly over
+// each 32 accumulators, the warps of a block in order, and the blocks' partial sums by 32 lanes
+// and a butterfly.  Results (and with them the rounding of the BF16 preconditioner's inputs) do
 // not depend on how many accumulators a thread holds.
 
 // pass 3 (marked vectors only): partial dots <V_j, u> of the new vector u, reduced by the
@@ -90,8 +89,9 @@ __global__ void k_reduce_dots(const double* __restrict__ part, int nblk, int nk,
 // subtracts h2_0 v_0 from u (see subtract_sparse_v0), in place of the update pass.
 template <int KP, bool ZS = false>
 __global__ void __launch_bounds__(kThreads)
-k_reorth_dots(double* u, const double* __restrict__ V, size_t vstride, size_t n2, int nk, double* __restrict__ part, int nblk,
-              const VecCtl* __restrict__ ctl, unsigned int* cnt, double* h2, int ncols) {
+k_reorth_dots(double* u, const double* __restrict__ V, size_t vstride, size_t n2, int nk,
+              double* __restrict__ part, int nblk, const VecCtl* __restrict__ ctl,
+              unsigned int* cnt, double* h2, int ncols) {
   const int b = blockIdx.y;
   if (!ctl[b].gm_active || !ctl[b].reorth) return;
   double* ub = u + (size_t)b * vstride;

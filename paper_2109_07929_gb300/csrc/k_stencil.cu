@@ -759,7 +759,10 @@ __device__ __forceinline__ int half_scatter_index(int lane) {
 // HBM below.  1024 x 1024, 16 vectors, nk = 1: 170 us one cell per thread, 157 us in pairs;
 // 256 x 256, 8 vectors, first step: 13.0 and 8.7 us.
 // KP >= nk accumulators; exact up to nk = 8, because an FMA predicated off still takes its
-// turn on the FP64 pipe (1024 x 1024, 16 vectors, nk = 3: 329 us with four, 264 with three).
+// turn on the FP64 pipe (1024 x 1024, 16 vectors, nk = 3: 329 us with four, 264 with three);
+// beyond that within a fifth or so, in steps of 2, 4 and 8 (30 applies of a cycle, Jacobi
+// preconditioner: 1024 x 1024, 4 vectors 12.1 ms, with 16 and 32 alone 12.6; 512 x 512, one
+// vector 1.34 and 1.38).
 template <int KP, typename ZT, int AM, bool ZS, int W>
 __global__ void __launch_bounds__(kThreads)
 k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
@@ -778,7 +781,8 @@ k_spmv_dots(Grid gr, const double* __restrict__ D, const ZT* __restrict__ z,
   double* wt = w + (size_t)b * n2;
   double* wb = wt + mn;
   const double* Vb_ = V + (size_t)b * vstride;
-  constexpr int KPP = KP <= 1 ? 1 : (KP <= 2 ? 2 : (KP <= 4 ? 4 : (KP <= 8 ? 8 : (KP <= 16 ? 16 : 32))));
+  constexpr int KPP =
+      KP <= 1 ? 1 : (KP <= 2 ? 2 : (KP <= 4 ? 4 : (KP <= 8 ? 8 : (KP <= 16 ? 16 : 32))));
   double acc[W][KPP] = {};
   const int half = (W == 2) ? (int)threadIdx.x / (kThreads / 2) : 0;
   const int vb = W * blockIdx.x + half;                 // block of the summation
