@@ -295,9 +295,10 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUten
 // 128 x N x 16 into one of two accumulators, and 8 warps drain the other one, 64 pixels at a
 // time.  The input rows go through 16-byte asynchronous copies: a TMA box of one 8-channel
 // plane consists of 16-byte rows, and 700 of those per stage took three times its MMAs.
-// Bound: the input rows' copies and the drain, each about 1200 clocks per stage against 430
-// of MMAs.  32 images of 256 x 256, 11 x 11, dilation 4: 1495 us, now 775 (one CTA per tile
-// with the drain exposed: 1081; persistent with TMA input rows: 828).
+// Bound: no unit (tensor pipe active 31 %, L2 56 %), but the chain of a stage, copy, landing,
+// MMAs and release: about 1300 clocks a stage against 430 of MMAs.  32 images of 256 x 256, 11 x
+// 11, dilation 4: 1495 us, now 775 (one CTA per tile with the drain exposed: 1081; persistent with
+// TMA input rows: 828).
 constexpr int kTapM = 4;               // taps per M tile
 constexpr int kTapPad = 36;            // floats per pixel of the epilogue's staging rows
 constexpr int kTapChunk = 64;          // pixels drained at a time
@@ -826,7 +827,7 @@ k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // ---- weight gradient, rows against rows --------------------------------------------------
 //
 // k_conv_wgrad_tc brings 20 KB through shared memory per 64 pixels for 4 MMAs of 16 clocks'
-// work: it is bound by L2 reads (201 TFLOP/s).  Here a CTA owns one kernel column kx and
+// work (201 TFLOP/s).  Here a CTA owns one kernel column kx and
 // multiplies 4 gradient rows y + j d (M = 4 x 32 output channels) by the K + 3 input rows
 // y + (i - r) d shifted by (kx - r) d pixels (N = 32 (K + 3) input channels, at most the 512
 // TMEM columns):
@@ -837,8 +838,8 @@ k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // partial sum per CTA.  Gradient rows beyond the image, where the row blocks do not divide H,
 // are kept out of D by the MMA's lane mask and not only by their zeros, which an infinity or a
 // NaN in x would turn into NaN; D starts from zeros, so that every MMA can have a mask.
-// Bound: L2 reads and MMA issue.  32 images of 256 x 256, 11 x 11, dilation 4, with the sums
-// behind it: 2779 us per call, now 685.
+// Bound: the stages in flight, three of 72 KB (tensor pipe active 42 %, L2 41 %).  32 images of
+// 256 x 256, 11 x 11, dilation 4, with the sums behind it: 2779 us per call, now 687.
 constexpr int kWrJ = 4;                                 // gradient rows per CTA step
 constexpr int kWrRow = kWgPix * kC * 2;                 // 64 pixels of a row: 4 KB
 constexpr int kWrMaxK = 512 / kC - (kWrJ - 1);          // 13

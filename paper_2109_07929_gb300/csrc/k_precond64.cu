@@ -27,8 +27,8 @@
 // none, where a chain of FMAs keeps 53 of each and rounds at 2^-53 of its partial sums.  The
 // apply's error in the norm falls all the same (96 x 160 to 40 x 600, random, spike, one-column,
 // graded, decaying and smooth right-hand sides, a from 2e-5 to 5: 2.7e-16 to 8.2e-16 of |z|, the
-// chain's 7.2e-16 to 2.1e-15); single small components move both ways, a spike's far field and
-// the largest of a smooth z's by up to 6 times the chain's error, others below it.
+// chain's 7.2e-16 to 2.1e-15); single components move both ways: in a spike's far field and a
+// few of a smooth z up to 6 times the chain's error, most others below it.
 // One apply (four transforms), against the FMA kernel: 512 x 512, 4 vectors 520 us (8300),
 // 1024 x 1024 933 us (16500), 64 x 64 135 us (324), 16 x 16 110 us (126).
 #include <cuda.h>
@@ -171,7 +171,8 @@ struct OzArgs {
 // One 128 x 64 output tile per CTA: 8 accumulators (one per weight) fill the TMEM; thread 0
 // streams both operands' 8 slices with one TMA box each (96 KB per 32 of K, two stages),
 // thread 32 issues the 36 slice products of a stage, and the 8 warps join the accumulators.
-// Bound: shared-memory reads of the operands (N = 64: 6 KB per MMA of 32 clocks' work).
+// Bound: shared-memory reads of the operands (N = 64: 6 KB per MMA of 32 clocks' work; 512 x 512,
+// 4 vectors: 65 % of their rate, the tensor pipe active 35 %) and a second wave two thirds full.
 // ADD: a later K range, added to O.
 template <bool ADD>
 __global__ void __launch_bounds__(kOzThreads, 1)

@@ -25,9 +25,9 @@
 // against 3, with 32 times the threads.  All products are of factors 0 < q < 1, so nothing
 // is amplified.  The factors depend on a only and are built once per GMRES cycle, in closed
 // form.
-// Bound: the FP64 pipe (13 instructions per cell).  1024 x 1024, 4 vectors, per apply: 1330
-// us (factor 460, columns 502, rows 273, stencils 97), now 115 (51 and 64) and the factors 30 us
-// once per cycle.
+// Bound: the FP64 pipe (13 instructions per cell; busy 79 % in the columns, 82 % in the rows).
+// 1024 x 1024, 4 vectors, per apply: 1330 us (factor 460, columns 502, rows 273, stencils 97),
+// now 115 (51 and 64) and the factors 30 us once per cycle.
 #include "mca_internal.cuh"
 
 namespace mca {
