@@ -1267,6 +1267,16 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     return MCA_ERR_CUDA;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // what k_conv_tc's stages hold is what a layer may ask for, whichever form runs: a row segment
+  // takes 64 bytes per pixel, 128 + (K - 1) d of them (compared in 64 bits: the plan's own
+  // arithmetic has 32)
+  const bool fits = (int64_t)(ksize - 1) * dilation <= 227 * 1024 / 64;
+  const ConvPlan plan = !fits ? ConvPlan{} : (cout_mma == 32) ? conv_plan<32>(ksize, dilation)
+                                                              : conv_plan<16>(ksize, dilation);
+  if (plan.stages < 2 || plan.smem > 227 * 1024) {
+    set_error_message("mca_cnn_conv: kernel size and dilation too large for one row segment");
+    return MCA_ERR_INVALID_ARG;
+  }
   TapPlan tp{};
   if (cout_mma == 32 && tap_plan(ksize, dilation, w, tp)) {
     CUtensorMap tmW;
@@ -1294,15 +1304,6 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     k_conv_taps<<<a.tiles < sms ? a.tiles : sms, kTapThreads, tp.smem, s>>>(tmW, a);
     count_launches(1);
     return launch_status("mca_cnn_conv launch");
-  }
-  // a row segment takes 64 bytes per pixel, 128 + (K - 1) d of them (compared in 64 bits: the
-  // plan's own arithmetic has 32)
-  const bool fits = (int64_t)(ksize - 1) * dilation <= 227 * 1024 / 64;
-  const ConvPlan plan = !fits ? ConvPlan{} : (cout_mma == 32) ? conv_plan<32>(ksize, dilation)
-                                                              : conv_plan<16>(ksize, dilation);
-  if (plan.stages < 2 || plan.smem > 227 * 1024) {
-    set_error_message("mca_cnn_conv: kernel size and dilation too large for one row segment");
-    return MCA_ERR_INVALID_ARG;
   }
   CUtensorMap tmX, tmW;
   if (!tc::make_map_nhwc32_k8(&tmX, x, w, h, n, plan.wbox) ||

@@ -171,3 +171,16 @@ def test_dilations_beyond_the_image(K, d):
         for dd in (d, 1431655721, 1431655722, 1431655766):
             assert mca.load().mca_cnn_conv(x.data_ptr(), N, H, W, wt.data_ptr(), K, dd, C, C, None, 0, 0,
                                            None, out.data_ptr(), None, None) == mca.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("K,most", [(3, 224), (5, 112), (7, 70), (9, 53), (11, 40), (13, 33), (15, 28)])
+def test_dilations_that_a_layer_may_ask_for(K, most):
+    """A convolution takes the dilations whose row segment k_conv_tc's stages hold, and refuses the
+    next one, whichever form runs."""
+    N, H, W = 1, 3, 20
+    x = torch.zeros(N, H, W, C, device=DEV).to(torch.bfloat16)
+    out, wt = torch.empty_like(x), torch.zeros(K * K, C, C, device=DEV).to(torch.bfloat16)
+    for d, rc in ((most, 0), (most + 1, mca.ERR_INVALID_ARG)):
+        assert mca.load().mca_cnn_conv(x.data_ptr(), N, H, W, wt.data_ptr(), K, d, C, C, None, 0, 0,
+                                       None, out.data_ptr(), None, None) == rc
+    assert mca.load().mca_cnn_check(None) == 0
