@@ -14,8 +14,8 @@
 //   forward  out[p][co] = sum_t sum_ci W[t][co][ci] x[p + off_t][ci].  k_conv_taps (32 output
 //            channels, K >= 5): four taps' weights are the rows (M = 4 x 32), the pixels of an
 //            input row the columns, and the drain adds the four taps' shifted rows.
-//            k_conv_tc (16 output channels, small kernels, dilations beyond k_conv_taps'
-//            shared memory): a CTA owns 128 pixels of one image row (M = 128, TMEM lane =
+//            k_conv_tc (16 output channels, small kernels, and where taps_faster finds it the
+//            faster one): a CTA owns 128 pixels of one image row (M = 128, TMEM lane =
 //            pixel) and all output channels (N = 16 or 32); per kernel row ky one pipeline
 //            stage holds the shifted input row segment (128 + (K - 1) d pixels, out-of-range
 //            pixels read as zero: the padding) in the K-major layout without swizzle, whose
@@ -315,7 +315,7 @@ struct TapPlan {
   int smem;
 };
 
-// False where the old form is the better one (or the only one that fits).
+// False where the form does not fit.
 bool tap_plan(int K, int d, int W, TapPlan& p) {
   if (K < 5) return false;             // a row of 1 or 3 taps would leave M mostly zero
   if (d > 256 / (kTapM - 1)) return false;             // (before the products below overflow)
@@ -344,6 +344,28 @@ bool tap_plan(int K, int d, int W, TapPlan& p) {
   if (p.stages < 2) return false;
   p.smem = p.stages * p.stage + kTapStaging + 512 + 1024;
   return true;
+}
+
+// Which form of a convolution is the faster one, by the time (us) that each takes on `sms` SMs,
+// fitted to 415 layers of 1 to 32 images (kernels 5 to 15, dilations up to where k_conv_tc ends;
+// mean error 9 % and 12 %).  k_conv_taps: its stages' bytes, for the kernel rows inside the image
+// (more where only two stages fit), and its drain per 64 pixels, over the waves of tiles; large
+// dilations leave few pixels of its 256 columns (1024 x 1024, K = 5: d = 32 256 us against 307,
+// d = 48 358 and 345, d = 70 1224 and 405), and one wave of wide tiles is mostly its pipeline's
+// start (17 x 500, 2 images, K = 5: 12.8 us against 8.9).  k_conv_tc: K stages per tile of 128
+// pixels, with the segment's length.  The line lies at 1.05, for the fit's own error: of the 415
+// layers, one is then slower than in k_conv_tc (12.4 against 10.7 us), 32 with k_conv_taps alone.
+bool taps_faster(const TapPlan& p, int n, int h, int w, int K, int d, int sms) {
+  const double images_rows = (double)n * h;
+  double inside = 0.0;                   // kernel rows inside the image, mean over its rows
+  for (int ky = 0; ky < K; ++ky) inside += std::max(0, h - std::abs(ky - K / 2) * d) / (double)h;
+  const double waves = std::ceil(images_rows * ((w + p.P - 1) / p.P) / sms);
+  const double waves_tc = std::ceil(images_rows * ((w + kPix - 1) / kPix) / sms);
+  const double kb = p.stage / 1024.0;
+  const double taps = 6.5 + waves * (inside * kb * (p.stages > 2 ? 0.0156 : 0.0258) +
+                                     0.8 * ((p.P + kTapChunk - 1) / kTapChunk)) + 0.23 * K;
+  const double tc = 4.8 + waves_tc * (K * (0.67 + 0.045 * K) + 0.010 * (K - 1) * d);
+  return 1.05 * taps <= tc;
 }
 
 struct TapArgs {
@@ -1277,8 +1299,14 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     set_error_message("mca_cnn_conv: kernel size and dilation too large for one row segment");
     return MCA_ERR_INVALID_ARG;
   }
+  int sms = 0;
+  if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
+    set_last_cuda_error(e, "mca_cnn_conv device", __FILE__, __LINE__);
+    return MCA_ERR_CUDA;
+  }
   TapPlan tp{};
-  if (cout_mma == 32 && tap_plan(ksize, dilation, w, tp)) {
+  if (cout_mma == 32 && tap_plan(ksize, dilation, w, tp) &&
+      taps_faster(tp, n, h, w, ksize, dilation, sms)) {
     CUtensorMap tmW;
     if ((reinterpret_cast<uintptr_t>(x) & 15) != 0 ||
         !tc::make_map_taps(&tmW, wt, ksize, kC, kTapM)) {
@@ -1296,11 +1324,6 @@ int mca_cnn_conv(const uint16_t* x, int32_t n, int32_t h, int32_t w, const uint1
     a.w = reinterpret_cast<const __nv_bfloat16*>(wt);
     a.plan = tp;
     a.tiles = n * h * a.xt;            // (n h w < 2^31)
-    int sms = 0;
-    if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
-      set_last_cuda_error(e, "mca_cnn_conv device", __FILE__, __LINE__);
-      return MCA_ERR_CUDA;
-    }
     k_conv_taps<<<a.tiles < sms ? a.tiles : sms, kTapThreads, tp.smem, s>>>(tmW, a);
     count_launches(1);
     return launch_status("mca_cnn_conv launch");

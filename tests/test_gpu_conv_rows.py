@@ -184,3 +184,34 @@ def test_dilations_that_a_layer_may_ask_for(K, most):
         assert mca.load().mca_cnn_conv(x.data_ptr(), N, H, W, wt.data_ptr(), K, d, C, C, None, 0, 0,
                                        None, out.data_ptr(), None, None) == rc
     assert mca.load().mca_cnn_check(None) == 0
+
+
+@pytest.mark.parametrize("K,d,N,H,W", [(5, 1, 2, 17, 500), (5, 20, 1, 33, 47), (5, 60, 1, 96, 130),
+                                       (7, 48, 2, 70, 60), (9, 53, 1, 64, 300), (15, 28, 1, 120, 70),
+                                       (11, 40, 3, 30, 41), (13, 20, 6, 21, 65), (5, 53, 9, 21, 70),
+                                       (11, 4, 2, 40, 150)])
+def test_layer_at_the_sizes_where_forms_change(K, d, N, H, W):
+    """Forward, backward data and weight gradient on both sides of the rules that choose a form:
+    dilations that leave few pixels of a tile, single waves, images of fewer rows than four
+    dilations.  FP32 sums of exact BF16 products: 1e-5 of the summed term magnitudes, BF16
+    outputs within 2^-8 of the value besides."""
+    g = torch.Generator(device=DEV).manual_seed(K * H + d)
+    x, gz = (torch.randn((N, H, W, C), generator=g, device=DEV).to(torch.bfloat16)
+             for _ in range(2))
+    w = (torch.randn((C, C, K, K), generator=g, device=DEV) / (C * K * K) ** 0.5)
+    w = w.to(torch.bfloat16).float()
+    got = [_convolve(x, w, d, torch.zeros(C, device=DEV)), _convolve(gz, w, d, backward_of=x),
+           _weight_gradient(x, gz, K, d)[0]]
+
+    def ref(xv, wv, gzv):
+        xv = xv.double().permute(0, 3, 1, 2).cpu().requires_grad_(True)
+        wv = wv.double().cpu().requires_grad_(True)
+        y = torch.nn.functional.conv2d(xv, wv, padding=d * (K // 2), dilation=d)
+        y.backward(gzv.double().permute(0, 3, 1, 2).cpu())
+        return [y.detach().permute(0, 2, 3, 1), xv.grad.permute(0, 2, 3, 1), wv.grad]
+
+    want, size = ref(x, w, gz), ref(x.abs(), w.abs(), gz.abs())
+    want[1] = torch.where(x.double().cpu() > 0, want[1], 0.1 * want[1])
+    for k in range(3):
+        half = 2.0 ** -8 * want[k].abs() if k < 2 else 0.0
+        assert bool(((got[k].double().cpu() - want[k]).abs() <= half + 1e-5 * size[k]).all())
