@@ -28,7 +28,8 @@
 //   weight gradient gW[t][co][ci] = sum_p gz[p][co] x[p + off_t][ci], K = pixels, both
 //            operands straight from the NHWC tensors as MN-major tiles.  k_wgrad_rows (K from 5
 //            to 13): rows of the gradient against rows of the input, all taps of a kernel row
-//            at once.  k_conv_wgrad_tc (the other kernel sizes): M = 4 taps x 32 input
+//            at once.  k_conv_wgrad_tc (the other kernel sizes, and where wgrad_rows_faster
+//            finds it the faster one): M = 4 taps x 32 input
 //            channels, N = 32 output channels, 64 consecutive pixels of a row per stage, a CTA
 //            covers one group of 4 taps over a block of rows.  Both write FP32 partial sums
 //            that a second kernel adds in a fixed order.
@@ -882,6 +883,45 @@ struct WrArgs {
   float* part;           // [chunk][t][ci 32][co 32]
 };
 
+struct WrPlan {
+  int blocks, nxc, items, chunks;
+};
+
+// nmax: partial sums that the scratch holds
+WrPlan wgrad_rows_plan(int n, int h, int w, int K, int d, int nmax, int sms) {
+  WrPlan p{};
+  const int64_t period = (int64_t)kWrJ * d;          // image rows of d row blocks
+  p.blocks = (int)(h / period * d + std::min<int64_t>(h % period, d));
+  p.nxc = (w + kWgPix - 1) / kWgPix;
+  p.items = n * p.blocks * p.nxc;
+  const int most = std::min(kWrItems, kWgRows * p.nxc);
+  p.chunks = (p.items + most - 1) / most;
+  // whole waves of CTAs (one resides per SM), two at least: 11 images of 187 x 187, dilation 8,
+  // 182 us per call with 33 chunks (2.4 waves), 158 with 41; 32 of 256 x 256, 717 and 685
+  const int waves = std::max(2, (K * p.chunks + sms - 1) / sms);
+  p.chunks = std::max(p.chunks, waves * sms / K);
+  p.chunks = std::min(p.chunks, std::min(nmax, p.items));
+  return p;
+}
+
+// Which form is the faster one, by the time (us) of each with its sums, fitted to 375 layers of 1
+// to 32 images (kernels 5 to 13; mean error 13 % and 16 %): the steps of k_wgrad_rows' waves
+// against the per-tap form's groups of four taps.  Images of fewer rows than four dilations leave
+// most of a row block's gradient rows outside (27 images of 21 x 169, K = 5, d = 53: 88 us against
+// 48; 12 of 12 x 15, K = 7, d = 32: 36 and 21).  The line lies at 1.1, for the fit's own error: of
+// the 375 layers, three are then slower than in the per-tap form, by 6 % at most, 53 with
+// k_wgrad_rows alone.
+bool wgrad_rows_faster(const WrPlan& p, int n, int h, int w, int K, int nmax, int sms) {
+  const int taps = K * K, steps = (p.items + p.chunks - 1) / p.chunks;
+  const int waves = (K * p.chunks + sms - 1) / sms;
+  const double rows = 13.7 + waves * (0.0577 * steps * (K + 7) + 0.296 * K) +
+                      0.0011 * p.chunks * taps;
+  const double share = (double)std::min<int64_t>(kWgRows, (int64_t)n * h) * p.nxc;
+  const double groups = (double)((taps + kWgTaps - 1) / kWgTaps) * nmax;
+  const double per_tap = 12.2 + share * (0.351 * groups / sms + 0.507) + 0.00164 * nmax * taps;
+  return 1.1 * rows <= per_tap;
+}
+
 __global__ void __launch_bounds__(128, 1)
 k_wgrad_rows(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG,
              WrArgs a) {
@@ -1383,28 +1423,21 @@ int mca_cnn_conv_wgrad(const uint16_t* x, const uint16_t* gz, int32_t n, int32_t
   // partial sums: the scratch holds one set per kWgRows image rows
   const int nmax = (int)(((int64_t)n * h + kWgRows - 1) / kWgRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  int sms = 0;
+  if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
+    set_last_cuda_error(e, "mca_cnn_conv_wgrad device", __FILE__, __LINE__);
+    return MCA_ERR_CUDA;
+  }
+  const WrPlan rp = wgrad_rows_plan(n, h, w, ksize, d, nmax, sms);
   int nchunk;
-  if (ksize >= 5 && ksize <= kWrMaxK) {
+  if (ksize >= 5 && ksize <= kWrMaxK && wgrad_rows_faster(rp, n, h, w, ksize, nmax, sms)) {
     WrArgs a{};
     a.H = h; a.K = ksize; a.d = d; a.r = (ksize - 1) / 2;
-    const int64_t period = (int64_t)kWrJ * d;          // image rows of d row blocks
-    a.blocks = (int)(h / period * d + std::min<int64_t>(h % period, d));
-    a.nxc = (w + kWgPix - 1) / kWgPix;
-    a.items = n * a.blocks * a.nxc;
+    a.blocks = rp.blocks;
+    a.nxc = rp.nxc;
+    a.items = rp.items;
     a.part = scratch;
-    int sms = 0;
-    if (const cudaError_t e = sm_count(&sms); e != cudaSuccess) {
-      set_last_cuda_error(e, "mca_cnn_conv_wgrad device", __FILE__, __LINE__);
-      return MCA_ERR_CUDA;
-    }
-    const int most = std::min(kWrItems, kWgRows * a.nxc);
-    nchunk = (a.items + most - 1) / most;
-    // whole waves of CTAs (one resides per SM), two at least: 11 images of 187 x 187, dilation
-    // 8, 182 us per call with 33 chunks (2.4 waves), 158 with 41; 32 of 256 x 256, 717 and 685
-    const int waves = std::max(2, (ksize * nchunk + sms - 1) / sms);
-    nchunk = std::max(nchunk, waves * sms / ksize);
-    if (nchunk > nmax) nchunk = nmax;
-    if (nchunk > a.items) nchunk = a.items;
+    nchunk = rp.chunks;
     const int stage = (ksize + 2 * kWrJ - 1) * kWrRow;
     a.stages = kWrStages * stage <= 224 * 1024 ? kWrStages : 2;
     const int smem = a.stages * stage + 512 + 1024;
