@@ -984,17 +984,22 @@ bool in_pairs(const Grid& gr, const double* D, const ZT* z, size_t zstride, cons
          (zstride & 1) == 0 && (vstride & 1) == 0;
 }
 
-// z: the vector of batch entry 0, later entries zstride apart
+// z: the vector of batch entry 0, later entries zstride apart.  Pairs of cells in FP32 and its
+// pairs (1024 x 1024, 3 vectors, FP32: 28 us per call, one cell per thread 30); in FP64 they
+// only wait longer for their loads (67 us, one cell per thread 61; FP64 on FP32 z 79 and 73).
 template <typename ZT, int AM>
 void apply_only(const Grid& gr, const double* D, const ZT* z, size_t zstride, double* w, int nblk,
                 int B, cudaStream_t s) {
   const FastDiv by_n(gr.n);
-  if (in_pairs(gr, D, z, zstride, w, nullptr, 0))
-    k_spmv_dots<1, ZT, AM, false, 2><<<dim3((nblk + 1) / 2, B), kThreads, 0, s>>>(
-        gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
-  else
-    k_spmv_dots<1, ZT, AM, false, 1><<<dim3(nblk, B), kThreads, 0, s>>>(
-        gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
+  if constexpr (AM != kApplyF64) {
+    if (in_pairs(gr, D, z, zstride, w, nullptr, 0)) {
+      k_spmv_dots<1, ZT, AM, false, 2><<<dim3((nblk + 1) / 2, B), kThreads, 0, s>>>(
+          gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
+      return;
+    }
+  }
+  k_spmv_dots<1, ZT, AM, false, 1><<<dim3(nblk, B), kThreads, 0, s>>>(
+      gr, D, z, zstride, w, nullptr, 0, 0, nullptr, nblk, nullptr, nullptr, nullptr, by_n);
 }
 
 // V: basis vector 0 of batch entry 0 (nk vectors N2 apart, entries vstride apart)
