@@ -135,8 +135,8 @@ def _solve_line(d, g, w):
     return y
 
 
-@pytest.mark.parametrize("m,n", [(2, 2), (1, 31), (32, 33), (65, 2), (100, 1025), (2049, 3),
-                                 (1057, 40)])
+@pytest.mark.parametrize("m,n", [(2, 2), (8, 9), (9, 8), (1, 31), (32, 33), (65, 2), (100, 1025),
+                                 (2049, 3), (1057, 40)])
 def test_mhat_solves_are_backward_stable(m, n):
     """G_2 z_b = r_b and z_t G_1 = r_t + a z_b to rounding, for a / g on both sides of the closed
     form's two branches and at both ends.  A chunk of L nodes forms its carries' factors as
